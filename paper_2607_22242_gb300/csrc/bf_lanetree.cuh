@@ -44,13 +44,12 @@
 //     lane; roots come from a per-block counter in shared memory (in the
 //     one-scenario search, once the block's share is gone, from a counter in
 //     device memory);
-//   * a checkpoint is nine state words (eleven in the wide form): the
+//   * a checkpoint is nine state words (twelve in the wide form): the
 //     per-tool words of the tools running at it are never written again
 //     while it can still be resumed.
 // Arithmetic is that of bf_sim.cuh: u32 real time, virtual clock modulo 2^32,
 // GPU completion ceil(rem * f[k] / 2^20), the CPU-event advance
-// floor(dt * 2^20 / f[k]) by the per-k reciprocal of Granlund and Montgomery
-// (PLDI 1994, Thm 4.2).
+// floor(dt * 2^20 / f[k]) by a per-k reciprocal (cpu_advance).
 #pragma once
 
 #include <stdint.h>
@@ -68,8 +67,8 @@ constexpr uint32_t kLtPartTools = 4;    // tools per table-driven part of the mo
 constexpr uint32_t kLtPartCombos = 81;  // 3^kLtPartTools
 constexpr uint32_t kLtRootParts = 4;    // root tools [0,4), [4,8), [8,12), [12,x)
 constexpr uint32_t kLtParts = kLtRootParts + 2;  // the root's parts, level [x,y), level [y,n)
-constexpr uint32_t kLtStateWords = 9;   // pend, run, qset, qlist (2 words), T, V, tc, gm
-constexpr uint32_t kLtWideStateWords = 11;  // and the wide queue's second word (2 words)
+constexpr uint32_t kLtStateWords = 9;   // pend and run (16 bits each), qset, qlist (2 words), T, V, tc, gm, tx
+constexpr uint32_t kLtWideStateWords = 12;  // pend and run apart, and the wide queue's second word (2 words)
 
 // State words of a checkpoint in the narrow (W = false) or wide form.
 template <bool W>
@@ -90,8 +89,7 @@ struct LaneTreeRecord {
   uint32_t vram[kLtMaxTools];
   uint32_t pv[kLtMaxTools];      // canonical place value 3^orig of each tool
   uint32_t f[kLtMaxTools + 1];
-  uint32_t fshift[kLtMaxTools + 1];
-  uint64_t fmagic[kLtMaxTools + 1];
+  uint64_t frecip[kLtMaxTools + 1];  // floor(2^52 / f[k]) (cpu_advance)
 };
 
 // Per block: the record and the tables derived from it; NC 6-bit chunks
@@ -101,6 +99,7 @@ struct LtSharedT {
   LaneTreeRecord rec;
   uint32_t rt[NC][kLtChunk];  // rt[c][v]: tools whose predecessors in chunk c are all in v
   uint32_t lv[NC][kLtChunk];  // lv[c][v]: VRAM of the tools of chunk c in v
+  uint32_t qw[NC][kLtChunk];  // qw[c][v]: isolated gpu_queue times (us) of the tools of chunk c in v, summed
   // Mode combinations of the parts (see kLtParts): now / queue masks and the
   // canonical index part of combination j of each part.
   uint32_t cnow[kLtParts][kLtPartCombos];
@@ -121,6 +120,7 @@ struct LtState {
   uint32_t T, V;   // real time (us); virtual GPU clock (1/1024 us of isolated work, modulo 2^32)
   uint32_t tc;     // earliest end of a running CPU tool (0xFFFFFFFF if none)
   uint32_t gm;     // end stamp of the running GPU tool that ends first (when one runs)
+  uint32_t tx;     // latest end of any CPU tool started so far (0 if none; at most T once it has ended)
 };
 
 // Rows of one lane ([row][thread], `stride` threads): the per-tool words
@@ -141,11 +141,13 @@ __device__ __forceinline__ uint32_t lt_ready(const LtSharedT<NC>& S, uint32_t pe
   return r;
 }
 
+// The sum of a per-tool quantity over the tools of `set`, from its chunk
+// table (LtSharedT::lv: VRAM, LtSharedT::qw: gpu_queue times).
 template <uint32_t NC>
-__device__ __forceinline__ uint32_t lt_vram(const LtSharedT<NC>& S, uint32_t gpu_running) {
+__device__ __forceinline__ uint32_t lt_sum(const uint32_t (&table)[NC][kLtChunk], uint32_t set) {
   uint32_t m = 0u;
 #pragma unroll
-  for (uint32_t c = 0; c < NC; ++c) m += S.lv[c][(gpu_running >> (kLtChunkBits * c)) & (kLtChunk - 1u)];
+  for (uint32_t c = 0; c < NC; ++c) m += table[c][(set >> (kLtChunkBits * c)) & (kLtChunk - 1u)];
   return m;
 }
 
@@ -155,13 +157,17 @@ __device__ __forceinline__ void lt_fill_tables(LtSharedT<NC>& S) {
   const LaneTreeRecord& R = S.rec;
   for (uint32_t e = threadIdx.x; e < NC * kLtChunk; e += blockDim.x) {
     const uint32_t c = e / kLtChunk, v = e % kLtChunk, lo = kLtChunkBits * c;
-    uint32_t ready = 0u, mem = 0u;
+    uint32_t ready = 0u, mem = 0u, qus = 0u;
     for (uint32_t t = 0; t < R.n; ++t) {
       if ((((R.pred[t] >> lo) & (kLtChunk - 1u)) & ~v) == 0u) ready |= 1u << t;
-      if (t >= lo && t < lo + kLtChunkBits && ((v >> (t - lo)) & 1u)) mem += R.vram[t];
+      if (t >= lo && t < lo + kLtChunkBits && ((v >> (t - lo)) & 1u)) {
+        mem += R.vram[t];
+        qus += R.dur[2][t] >> 10;
+      }
     }
     S.rt[c][v] = ready;
     S.lv[c][v] = mem;
+    S.qw[c][v] = qus;
   }
   // Parts: root tools [0, min(x,4)), [4, min(x,8)), [8, min(x,12)), [12, x);
   // level tools [x, y), [y, n).
@@ -186,13 +192,13 @@ __device__ __forceinline__ void lt_fill_tables(LtSharedT<NC>& S) {
   }
   if (threadIdx.x == 0) {
     uint32_t* w = S.ck0;
-    w[0] = R.all_mask;        // pend: every tool
-    w[1] = w[2] = 0u;         // run, qset
-    w[3] = w[4] = 0u;         // qlist
-    w[5] = w[6] = 0u;         // T, V
-    w[7] = 0xFFFFFFFFu;       // tc: no CPU tool runs
-    w[8] = 0u;                // gm
-    w[9] = w[10] = 0u;        // the wide queue's second word
+    w[0] = R.all_mask;                  // pend: every tool (run, in its upper half when narrow: none)
+    w[1] = w[2] = w[3] = 0u;            // qset, qlist
+    w[4] = w[5] = 0u;                   // T, V
+    w[6] = 0xFFFFFFFFu;                 // tc: no CPU tool runs
+    w[7] = 0u;                          // gm
+    w[8] = 0u;                          // tx: no CPU tool has started
+    w[9] = w[10] = w[11] = 0u;          // wide: run, the queue's second word
   }
 }
 
@@ -201,9 +207,26 @@ enum LtStep : uint32_t { kLtContinue = 0, kLtFinished = 1, kLtInfeasible = 2, kL
 // One step of a lane's simulation under modes (now, que; the other tools run
 // on the CPU): the admission at T -- or kLtStopped, before it, when a tool of
 // `stop` would become ready -- then the next event and the retirements at it.
-// Returns kLtFinished once every tool has ended (the makespan is s.T).  The
-// loops' bodies are written as selects: lanes of a warp are at different
-// points of their simulations, and a branch in a body would run both sides.
+// Returns kLtFinished once the makespan is known, in s.T: when every tool has
+// ended, or in closed form as soon as no tool is pending and at most one GPU
+// tool runs.  The loops' bodies are written as selects: lanes of a warp are at
+// different points of their simulations, and a branch in a body would run both
+// sides.
+//
+// The closed form.  With no tool pending nothing but the queue can start any
+// more, and queued tools run one at a time.  While one GPU tool runs alone the
+// model's arithmetic has no rounding to reproduce event by event: f[1] = 1024,
+// so a CPU event dt later advances V by exactly dt * 1024, and the tool ends
+// at T + ceil(rem / 1024) whichever CPU tools end before it.  Work amounts are
+// whole microseconds (multiples of 1024 units), so each waiting tool then adds
+// its isolated time exactly, in any order; with nothing else on the GPU it
+// fits unless it is larger than M, which makes the mapping infeasible.  CPU
+// tools end at their fixed times, the latest of which is tx.  Steps are what
+// the kernels' issue slots go to: on the host emulator the closed form takes
+// the 16-tool layered workload from 2.28 to 0.90 steps per mapping and the
+// batch workload from 3.05 to 2.20.  Measured: 16-tool full search 1.59 -> 0.97 ms,
+// an 18-tool layered one 10.8 -> 6.2 ms, batch call of 4096 x 3^10 12.7 ->
+// 11.6 ms.
 template <uint32_t NC, bool W = false>
 __device__ __forceinline__ uint32_t lt_step(const LtSharedT<NC>& S, LtState& s, uint32_t now, uint32_t que,
                                             uint32_t stop, uint32_t* e, uint32_t stride) {
@@ -224,6 +247,7 @@ __device__ __forceinline__ uint32_t lt_step(const LtSharedT<NC>& S, LtState& s, 
       const bool first = isn && (!(s.run & gpu) || w < s.gm - s.V);
       s.gm = first ? val : s.gm;
       s.tc = isn ? s.tc : min(s.tc, val);
+      s.tx = (isn || s.tx > val) ? s.tx : val;
       s.run |= 1u << i;
     }
     // queued: join the FIFO in index order (a row is written when the tool starts)
@@ -239,14 +263,14 @@ __device__ __forceinline__ uint32_t lt_step(const LtSharedT<NC>& S, LtState& s, 
       }
       s.qset |= 1u << i;
     }
-    if ((ready & now) && lt_vram(S, s.run & gpu) > R.budget) return kLtInfeasible;  // out of memory
+    if ((ready & now) && lt_sum(S.lv, s.run & gpu) > R.budget) return kLtInfeasible;  // out of memory
   }
   // ---- queue head: the first tool of the FIFO --------------------------------
   if (s.qset && !(s.run & que)) {
     const uint32_t h = (uint32_t)(s.qlist & (W ? 31u : 15u)), hb = 1u << h;
     if (hb & R.big_mask) return kLtInfeasible;  // a head larger than M can never start
     const uint32_t rg = s.run & gpu;
-    if (lt_vram(S, rg | hb) <= R.budget) {  // no bypass: otherwise the head waits
+    if (lt_sum(S.lv, rg | hb) <= R.budget) {  // no bypass: otherwise the head waits
       const uint32_t w = R.dur[2][h], val = s.V + w;
       s.gm = (!rg || w < s.gm - s.V) ? val : s.gm;
       e[h * stride] = val;
@@ -261,33 +285,50 @@ __device__ __forceinline__ uint32_t lt_step(const LtSharedT<NC>& S, LtState& s, 
     }
   }
   // ---- next event -----------------------------------------------------------
-  const uint32_t rg = s.run & gpu;
-  const uint32_t k = __popc(rg), kk = k ? k : 1u;  // kk: a valid table index when no GPU tool runs
-  const uint32_t rem = s.gm - s.V;
-  const uint64_t tg = (uint64_t)s.T + (((uint64_t)rem * R.f[kk] + 0xFFFFFull) >> 20);
-  const bool gpu_event = k != 0u && tg <= (uint64_t)s.tc;
-  const uint32_t adv = (uint32_t)(__umul64hi(R.fmagic[kk], (uint64_t)(s.tc - s.T) << 20) >> R.fshift[kk]);
-  s.V = gpu_event ? s.gm : (k ? s.V + adv : s.V);
-  s.T = gpu_event ? (uint32_t)tg : s.tc;
-  // ---- retire everything that ends at T; the next CPU end and GPU stamp -----
-  // Only tools of the kinds that can end now are scanned: CPU tools when T
-  // reached the earliest CPU end, GPU tools at a GPU event (at a CPU event V
-  // stays below every running GPU tool's stamp); the other kind's earliest
-  // end is unchanged.
-  const bool cpu_event = s.tc == s.T;
-  uint32_t ntc = cpu_event ? 0xFFFFFFFFu : s.tc, nrem = gpu_event ? 0xFFFFFFFFu : s.gm - s.V, ended = 0u;
-  for (uint32_t m = (cpu_event ? s.run & ~gpu : 0u) | (gpu_event ? rg : 0u); m; m &= m - 1u) {
-    const uint32_t i = __ffs(m) - 1u, b = 1u << i, end = e[i * stride];
-    const bool isc = (gpu & b) == 0u;
-    const bool hit = end == (isc ? s.T : s.V);
-    ended |= hit ? b : 0u;
-    ntc = (isc && !hit) ? min(ntc, end) : ntc;
-    nrem = (!isc && !hit) ? min(nrem, end - s.V) : nrem;
+  uint32_t rg = s.run & gpu, k = __popc(rg);
+  const bool settled = s.pend == 0u && k <= 1u;  // the closed form applies at once
+  if (!settled) {
+    const uint32_t kk = k ? k : 1u;  // a valid table index when no GPU tool runs
+    const uint32_t rem = s.gm - s.V, dtc = s.tc - s.T, f = R.f[kk];
+    // The time to the next GPU end, rem * f / 2^20 rounded up, is below 2^29.
+    const uint32_t dtg = (uint32_t)(((uint64_t)rem * f + 0xFFFFFull) >> 20);
+    const bool gpu_event = k != 0u && dtg <= dtc;
+    const uint32_t adv = cpu_advance(dtc, f, R.frecip[kk]);
+    s.V = gpu_event ? s.gm : (k ? s.V + adv : s.V);
+    s.T = gpu_event ? s.T + dtg : s.tc;
+    // ---- retire everything that ends at T; the next CPU end and GPU stamp ---
+    // Only tools of the kinds that can end now are scanned: CPU tools when T
+    // reached the earliest CPU end, GPU tools at a GPU event (at a CPU event V
+    // stays below every running GPU tool's stamp); the other kind's earliest
+    // end is unchanged.
+    const bool cpu_event = s.tc == s.T;
+    uint32_t ntc = cpu_event ? 0xFFFFFFFFu : s.tc, nrem = gpu_event ? 0xFFFFFFFFu : s.gm - s.V, ended = 0u;
+    for (uint32_t m = (cpu_event ? s.run & ~gpu : 0u) | (gpu_event ? rg : 0u); m; m &= m - 1u) {
+      const uint32_t i = __ffs(m) - 1u, b = 1u << i, end = e[i * stride];
+      const bool isc = (gpu & b) == 0u;
+      const bool hit = end == (isc ? s.T : s.V);
+      ended |= hit ? b : 0u;
+      ntc = (isc && !hit) ? min(ntc, end) : ntc;
+      nrem = (!isc && !hit) ? min(nrem, end - s.V) : nrem;
+    }
+    s.run &= ~ended;
+    s.tc = ntc;
+    s.gm = s.V + nrem;
+    rg = s.run & gpu;
+    k = __popc(rg);
   }
-  s.run &= ~ended;
-  s.tc = ntc;
-  s.gm = s.V + nrem;
-  return (s.pend | s.run | s.qset) == 0u ? kLtFinished : kLtContinue;
+  // ---- the closed form --------------------------------------------------------
+  // After an event it must not pass by a queue head that could start beside the
+  // one running gpu_now tool (the next step decides that).
+  if (s.pend == 0u && k <= 1u && (settled || k == 0u || s.qset == 0u || (rg & que))) {
+    if (s.qset & R.big_mask) return kLtInfeasible;
+    const uint32_t rem = s.gm - s.V;
+    const uint32_t left = k ? (rem >> 10) + ((rem & 1023u) ? 1u : 0u) : 0u;
+    const uint32_t gpu_end = s.T + left + lt_sum(S.qw, s.qset);
+    s.T = s.tx > gpu_end ? s.tx : gpu_end;
+    return kLtFinished;
+  }
+  return kLtContinue;
 }
 
 // One lane's share of the block's roots: every mapping below each root it
@@ -338,31 +379,39 @@ __device__ __forceinline__ void lt_lane(const LtSharedT<NC>& S, uint32_t* rows, 
       }
       uint32_t* const cw = rows + (L == 2u ? n + SW : n) * stride;  // checkpoint L's state words
       if (descend) {  // save the state words
-        cw[0] = s.pend;
-        cw[stride] = s.run;
-        cw[2u * stride] = s.qset;
-        cw[3u * stride] = (uint32_t)s.qlist;
-        cw[4u * stride] = (uint32_t)(s.qlist >> 32);
-        cw[5u * stride] = s.T;
-        cw[6u * stride] = s.V;
-        cw[7u * stride] = s.tc;
-        cw[8u * stride] = s.gm;
+        cw[0] = W ? s.pend : s.pend | (s.run << 16);
+        cw[stride] = s.qset;
+        cw[2u * stride] = (uint32_t)s.qlist;
+        cw[3u * stride] = (uint32_t)(s.qlist >> 32);
+        cw[4u * stride] = s.T;
+        cw[5u * stride] = s.V;
+        cw[6u * stride] = s.tc;
+        cw[7u * stride] = s.gm;
+        cw[8u * stride] = s.tx;
         if (W) {
-          cw[9u * stride] = (uint32_t)s.qhi;
-          cw[10u * stride] = (uint32_t)(s.qhi >> 32);
+          cw[9u * stride] = s.run;
+          cw[10u * stride] = (uint32_t)s.qhi;
+          cw[11u * stride] = (uint32_t)(s.qhi >> 32);
         }
       } else {  // load a checkpoint's state words, or the time-0 state for a root
         const uint32_t* w = L == 0u ? S.ck0 : cw;
         const uint32_t ws = L == 0u ? 1u : stride;
         s.pend = w[0];
-        s.run = w[ws];
-        s.qset = w[2u * ws];
-        s.qlist = (uint64_t)w[3u * ws] | ((uint64_t)w[4u * ws] << 32);
-        s.T = w[5u * ws];
-        s.V = w[6u * ws];
-        s.tc = w[7u * ws];
-        s.gm = w[8u * ws];
-        if (W) s.qhi = (uint64_t)w[9u * ws] | ((uint64_t)w[10u * ws] << 32);
+        if (!W) {
+          s.run = s.pend >> 16;
+          s.pend &= 0xFFFFu;
+        }
+        s.qset = w[ws];
+        s.qlist = (uint64_t)w[2u * ws] | ((uint64_t)w[3u * ws] << 32);
+        s.T = w[4u * ws];
+        s.V = w[5u * ws];
+        s.tc = w[6u * ws];
+        s.gm = w[7u * ws];
+        s.tx = w[8u * ws];
+        if (W) {
+          s.run = w[9u * ws];
+          s.qhi = (uint64_t)w[10u * ws] | ((uint64_t)w[11u * ws] << 32);
+        }
       }
       // Modes and index part of the new job's level: a root's four table
       // parts (base-81 digits of the root), or one level combination (the

@@ -46,16 +46,11 @@ inline void build_tables(const bf_scenario_desc* d, bfk::TablesT<CAP>* t) {
   for (uint32_t k = 1; k <= (uint32_t)CAP; ++k) {
     // Entries above n are never used; fill them with f[n] so every k is defined.
     const uint32_t f = d->slowdown_q10[k <= n ? k : n];
-    uint32_t l = 0;
-    while ((1u << l) < f) ++l;  // ceil(log2 f)
-    if (l < 12) l = 12;
-    const unsigned __int128 num = (unsigned __int128)1 << (52 + l);
     t->f[k] = f;
-    t->fshift[k] = l - 12;
-    t->fmagic[k] = (uint64_t)((num + f - 1) / f);
+    t->frecip[k] = (1ull << 52) / f;
   }
   t->f[0] = 1024;
-  t->fmagic[0] = 1ull << 54;
+  t->frecip[0] = 1ull << 42;
 }
 
 // Number of mid tools M of the pruned search's split (bf_search_pruned):
@@ -281,8 +276,7 @@ inline void plan_for(const bfk::Tables& t, const uint32_t* anc, const uint32_t* 
   w->relabeled = t.relabeled;
   for (uint32_t k = 0; k <= (uint32_t)bfk::kMaxTools; ++k) {
     w->f[k] = t.f[k];
-    w->fshift[k] = t.fshift[k];
-    w->fmagic[k] = t.fmagic[k];
+    w->frecip[k] = t.frecip[k];
   }
 }
 
@@ -370,8 +364,7 @@ inline void build_window(const bfk::TablesT<CAP>& t, uint32_t w0, bfk::TablesT<N
   w->relabeled = t.relabeled;
   for (uint32_t k = 0; k <= (uint32_t)NW; ++k) {
     w->f[k] = t.f[k];
-    w->fshift[k] = t.fshift[k];
-    w->fmagic[k] = t.fmagic[k];
+    w->frecip[k] = t.frecip[k];
   }
 }
 
@@ -721,8 +714,7 @@ inline void lanetree_record(const bf_scenario_desc* d, bfk::LaneTreeRecord* r, u
   }
   for (uint32_t j = 0; j <= bfk::kLtMaxTools; ++j) {
     r->f[j] = last.f[j];
-    r->fshift[j] = last.fshift[j];
-    r->fmagic[j] = last.fmagic[j];
+    r->frecip[j] = last.frecip[j];
   }
   if (min_roots == 0) {
     lanetree_split(view, &r->x, &r->y, &r->nblocks);

@@ -18,11 +18,8 @@
 //     work and eg[i] == V exactly when it ends.  `gmin` is the stamp of the
 //     running GPU tool that ends first; processor sharing runs every GPU tool
 //     at the same rate, so it only changes when GPU tools start or end.
-//   * The floor division of a CPU event, floor(dt * 2^20 / f[k]) with
-//     dt * 2^20 < 2^52, uses a per-k reciprocal (Granlund & Montgomery,
-//     "Division by invariant integers using multiplication", PLDI 1994,
-//     Thm 4.2): m = ceil(2^(52+l) / f), l = max(12, ceil(log2 f));
-//     q = umulhi(m, n) >> (l - 12).
+//   * The floor division of a CPU event, floor(dt * 2^20 / f[k]), multiplies
+//     by a per-k reciprocal and corrects the quotient (cpu_advance).
 //   * A queued tool with m > M can never start, so such a mapping is rejected
 //     before simulating (the verdict the model reaches when that tool becomes
 //     the queue head).
@@ -45,6 +42,20 @@ constexpr uint32_t kInfeasible = 0xFFFFFFFFu;
 // least one tool, so a correct simulation needs at most n events).  Scenario
 // validation keeps real makespans <= 0xFFFFFFFD, so this value never collides.
 constexpr uint32_t kStalled = 0xFFFFFFFEu;
+
+// floor(dt * 2^20 / f) for the virtual-clock advance over a CPU event dt us
+// away (the quotient fits 32 bits there: it is below the remaining work of a
+// running GPU tool); r = floor(2^52 / f), 1024 <= f <= 65536.  dt * r / 2^32
+// is below the exact quotient by less than dt / 2^32 < 1, so its floor is the
+// quotient or one less, and the remainder (below 2f, exact modulo 2^32) tells
+// which.  Two 32-bit multiplies for the quotient and one for the remainder; a
+// 64 x 64-bit high product by a rounded-up reciprocal took about twice as many
+// instructions.
+__device__ __forceinline__ uint32_t cpu_advance(uint32_t dt, uint32_t f, uint64_t r) {
+  const uint32_t q = dt * (uint32_t)(r >> 32) + (uint32_t)(((uint64_t)dt * (uint32_t)r) >> 32);
+  const uint32_t rest = (dt << 20) - q * f;
+  return q + (rest >= f ? 1u : 0u);
+}
 
 enum RunResult : uint32_t { kRunFinished = 0, kRunInfeasible = 1, kRunStopped = 2 };
 
@@ -71,8 +82,7 @@ struct TablesT {
   uint32_t orig[CAP];
   uint32_t relabeled;
   uint32_t f[CAP + 1];        // f[k]; f[0] unused
-  uint32_t fshift[CAP + 1];   // l - 12
-  uint64_t fmagic[CAP + 1];   // ceil(2^(52+l) / f[k])
+  uint64_t frecip[CAP + 1];   // floor(2^52 / f[k]) (cpu_advance)
 };
 using Tables = TablesT<kMaxTools>;
 
@@ -147,9 +157,8 @@ inline int bucket_for(uint32_t w) {
 // the per-k slowdown constants and the predecessor masks.
 template <int CAP>
 struct SmemTablesT {
-  uint64_t magic[CAP + 1];
+  uint64_t recip[CAP + 1];
   uint32_t f[CAP + 1];
-  uint32_t shift[CAP + 1];
   uint32_t pred[CAP];
 };
 using SmemTables = SmemTablesT<kMaxTools>;
@@ -157,9 +166,8 @@ using SmemTables = SmemTablesT<kMaxTools>;
 template <int CAP>
 __device__ __forceinline__ void load_smem_tables(const TablesT<CAP>& tb, SmemTablesT<CAP>& s) {
   for (int k = threadIdx.x; k <= CAP; k += blockDim.x) {
-    s.magic[k] = tb.fmagic[k];
+    s.recip[k] = tb.frecip[k];
     s.f[k] = tb.f[k];
-    s.shift[k] = tb.fshift[k];
     if (k < CAP) s.pred[k] = tb.pred[k];
   }
 }
@@ -345,15 +353,14 @@ __device__ __forceinline__ uint32_t run(State<NT>& s, const TB& tb, const SD& sd
     const uint32_t kk = min(k, (uint32_t)NT);  // k <= NT always; keeps indexing in bounds
     bool gpu_event = false;
     if (k) {
-      const uint32_t rem = s.gmin - s.V;
-      const uint64_t tg = (uint64_t)s.T + (((uint64_t)rem * sd.f[kk] + 0xFFFFFull) >> 20);
-      if (tg <= (uint64_t)s.tc) {
-        s.T = (uint32_t)tg;
+      const uint32_t rem = s.gmin - s.V, dtc = s.tc - s.T, f = sd.f[kk];
+      const uint32_t dtg = (uint32_t)(((uint64_t)rem * f + 0xFFFFFull) >> 20);  // below 2^29
+      if (dtg <= dtc) {
+        s.T += dtg;
         s.V = s.gmin;
         gpu_event = true;
       } else {
-        const uint64_t num = (uint64_t)(s.tc - s.T) << 20;
-        s.V += (uint32_t)(__umul64hi(sd.magic[kk], num) >> sd.shift[kk]);
+        s.V += cpu_advance(dtc, f, sd.recip[kk]);
         s.T = s.tc;
       }
     } else {
