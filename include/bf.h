@@ -145,7 +145,12 @@ BF_API int bf_destroy_scenario(bf_scenario* scn);
  * d_makespan[j] = makespan of mapping first+j (0xFFFFFFFF if infeasible),
  * d_feasible[j] = 1/0.  Both are caller-owned device arrays of >= count
  * elements.  Asynchronous on `cuda_stream`.  count == 0 is a no-op.
- * BF_ERANGE if first+count > 3^n; BF_EINVAL on NULL pointers. */
+ * BF_ERANGE if first+count > 3^n; BF_EINVAL on NULL pointers.
+ * A scenario whose DAG has barriers (every tool >= c waits for every tool < c)
+ * is a row of independent segments: a large evaluation simulates each
+ * segment's mappings into tables in the handle and writes every mapping's
+ * makespan as the sum of its segments'.  Such evaluations of one handle may
+ * overlap each other; a captured one never uses the tables. */
 BF_API int bf_eval_mappings(const bf_scenario* scn, uint64_t first, uint64_t count,
                      uint32_t* d_makespan, uint8_t* d_feasible, void* cuda_stream);
 
@@ -239,7 +244,11 @@ typedef struct bf_tree_stats {
  * flags: 0 or BF_TREE_NO_PRUNE (every mapping of the space is simulated:
  * full enumeration).  `stats` may be NULL.  Allocates level buffers in the
  * handle on first use (about 1.7 GB for 32 tools in the full space).  Blocks
- * until the result is on the host.  The whole search, not only each level
+ * until the result is on the host.  A pruned search of a scenario cut by
+ * barriers into segments of at most 13 tools (see bf_eval_mappings) enumerates
+ * each segment on its own instead, in one launch, and adds their optima up
+ * (bf_search_pruned does the same); its stats count the segments as nodes and
+ * their mappings as leaves.  The whole search, not only each level
  * step, is held to the wait limit (bf_set_wait_timeout_ms): past it the call
  * returns BF_ETIMEOUT (an unpruned full space of 28 or more tools takes
  * hours). */

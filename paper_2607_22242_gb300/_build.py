@@ -96,7 +96,7 @@ def build(force: bool = False, extra_flags=(), verbose: bool = False) -> str:
         obj = os.path.join(BUILD_DIR, f"bf_kernels_nw{nt}.o")
         jobs.append([cc, *ARCH, *NVCC_FLAGS, *extra_flags, f"-DBF_NW={nt}", "-c",
                      os.path.join(CSRC, "bf_kernels.cu"), "-o", obj])
-    for unit in ("bf_tree", "bf_lanetree", "bf_capi", "bf_capi_tree"):
+    for unit in ("bf_tree", "bf_lanetree", "bf_segments", "bf_capi", "bf_capi_tree"):
         jobs.append([cc, *ARCH, *NVCC_FLAGS, *extra_flags, "-c", os.path.join(CSRC, unit + ".cu"), "-o",
                      os.path.join(BUILD_DIR, unit + ".o")])
 

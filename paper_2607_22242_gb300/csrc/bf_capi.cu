@@ -81,6 +81,19 @@ cudaError_t lib_malloc_async(void** p, size_t bytes, cudaStream_t st) {
   return cudaMallocAsync(p, bytes, st);
 }
 
+// Every tool runs at most max(c, floor((l+g+x) f[n] / 1024) + n + 1) us, and
+// at every instant before the end some tool runs, so the sum bounds every
+// makespan.
+uint64_t makespan_bound(const bf_scenario_desc* d) {
+  uint64_t bound = 0;
+  for (uint32_t v = 0; v < d->n; ++v) {
+    const uint64_t w = (uint64_t)d->load_us[v] + d->gpu_us[v] + d->xfer_us[v];
+    const uint64_t gpu_bound = w * d->slowdown_q10[d->n] / 1024 + d->n + 1;
+    bound += d->cpu_us[v] > gpu_bound ? d->cpu_us[v] : gpu_bound;
+  }
+  return bound;
+}
+
 int validate(const bf_scenario_desc* d, const char* who) {
   if (!d) return fail(BF_EINVAL, "%s: desc is NULL", who);
   const uint32_t n = d->n;
@@ -105,15 +118,7 @@ int validate(const bf_scenario_desc* d, const char* who) {
       return fail(BF_EINVAL, "%s: slowdown_q10 decreases at k=%u", who, k);
     if (d->slowdown_q10[k] > 65536) return fail(BF_EINVAL, "%s: slowdown_q10[%u] > 65536", who, k);
   }
-  // Every tool runs at most max(c, floor((l+g+x) f[n] / 1024) + n + 1) us,
-  // and at every instant before the end some tool runs, so the sum bounds
-  // every makespan.
-  uint64_t bound = 0;
-  for (uint32_t v = 0; v < n; ++v) {
-    const uint64_t w = (uint64_t)d->load_us[v] + d->gpu_us[v] + d->xfer_us[v];
-    const uint64_t gpu_bound = w * d->slowdown_q10[n] / 1024 + n + 1;
-    bound += d->cpu_us[v] > gpu_bound ? d->cpu_us[v] : gpu_bound;
-  }
+  const uint64_t bound = makespan_bound(d);
   if (bound > 0xFFFFFFFDull)
     return fail(BF_EINVAL, "%s: makespan bound %llu does not fit in 32 bits", who, (unsigned long long)bound);
   return BF_OK;
@@ -328,7 +333,8 @@ void build_lanetree_records(const bf_scenario_desc* descs, const uint32_t* ids, 
   });
 }
 
-inline size_t align256(size_t x) { return (x + 255) / 256 * 256; }
+constexpr size_t align256(size_t x) { return (x + 255) / 256 * 256; }
+constexpr size_t kTableOffset = align256(sizeof(bf_scratch));  // the segments' tables, behind the scratch
 
 // Index-list evaluation: the 20-slot kernels up to 20 tools, the 32-slot one above.
 cudaError_t launch_list(const bf_scenario* scn, const uint64_t* idx, uint64_t count, uint32_t* ms, uint8_t* fe,
@@ -341,6 +347,27 @@ cudaError_t launch_list(const bf_scenario* scn, const uint64_t* idx, uint64_t co
   BF_DISPATCH(bfk::bucket_for(n), CALL)
 #undef CALL
   return e;
+}
+
+// Whether work put on `st` is being captured (or whether that cannot be told).
+bool is_capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &status) != cudaSuccess) {
+    cudaGetLastError();
+    return true;
+  }
+  return status != cudaStreamCaptureStatusNone;
+}
+
+// Whether an evaluation of `count` mappings of a scenario cut by barriers sums
+// them up from its segments' tables: always without tables to simulate, else
+// from 2^17 mappings on when the tables have at most half as many entries.
+// Below that the second launch costs more than it saves (whole call; a 12-tool
+// fan-out with one 10-tool segment: 1,000 mappings 33 against 29 us in the
+// general kernel, 30,000 mappings 34 against 31 us, 531,441 mappings 34 against
+// 50 us; 2^25 mappings of the 19-tool spine 47 us against 1.57 ms).
+bool sums_pay(const bf_scenario* scn, uint64_t count) {
+  return scn->seg.count != 0u && (scn->seg.tables == 0u || (count >= (1u << 17) && scn->seg.entries <= count / 2u));
 }
 
 // One launch of the search kernel -- or, for the whole space of a scenario
@@ -357,26 +384,49 @@ int run_search(const bf_scenario* scn, uint64_t first, uint64_t count, bf_result
   // scenario's numbering, in which an index range is a box of the split.
   const bool whole = first == 0 && count == pow3(scn->desc.n);
   if (whole && scn->lanetree) {
-    const cudaError_t e = bfk::launch_lanetree_single(&scn->d_scratch->lt, scn->desc.n, scn->lt_x, scn->lt_blocks,
-                                                      &scn->d_scratch->search, scn->d_host_search_key, st);
+    const cudaError_t e = bfk::launch_lanetree_single(&scn->d_scratch->launch.lt, scn->desc.n, scn->lt_x, scn->lt_blocks,
+                                                      &scn->d_scratch->launch.search, scn->d_host_search_key, st);
     if (e != cudaSuccess) return cuda_fail(e, who);
     const int rc = wait_stream(st, who);
     if (rc != BF_OK) return rc;
-    fill_result(*static_cast<volatile unsigned long long*>(&scn->h_scratch->search.key), scn->desc.n, first, out);
+    fill_result(*static_cast<volatile unsigned long long*>(&scn->h_scratch->launch.search.key), scn->desc.n, first, out);
     return BF_OK;
   }
   const bfk::Tables& tb = whole ? scn->rtables : scn->tables;
   const bfk::Tables& tw = whole ? scn->rwindow : scn->window;
   const bfk::Plan plan = make_plan(whole ? scn->rplan : scn->plan, first, count, kSearchTasks);
   cudaError_t e = cudaSuccess;
-#define CALL(NW) launch_search_nw##NW(tb, tw, plan, &scn->d_scratch->search, scn->d_host_search_key, st)
+#define CALL(NW) launch_search_nw##NW(tb, tw, plan, &scn->d_scratch->launch.search, scn->d_host_search_key, st)
   BF_DISPATCH(bfk::bucket_for(tw.n), CALL)
 #undef CALL
   if (e != cudaSuccess) return cuda_fail(e, who);
   const int rc = wait_stream(st, who);
   if (rc != BF_OK) return rc;
-  fill_result(*static_cast<volatile unsigned long long*>(&scn->h_scratch->search.key), scn->desc.n, first, out);
+  fill_result(*static_cast<volatile unsigned long long*>(&scn->h_scratch->launch.search.key), scn->desc.n, first, out);
   return BF_OK;
+}
+
+int segment_optimum(const bf_scenario* scn, uint32_t radix, bf_result* out, cudaStream_t st, const char* who) {
+  const cudaError_t e =
+      bfk::launch_segment_optimum(scn->seg, radix, &scn->d_scratch->launch.seg, scn->d_host_best, st);
+  if (e != cudaSuccess) return cuda_fail(e, who);
+  const int rc = wait_stream(st, who);
+  if (rc != BF_OK) return rc;
+  fill_best(*static_cast<volatile bfk::BestRecord*>(&scn->h_scratch->best), scn->desc.n, out);
+  return BF_OK;
+}
+
+void fill_best(const volatile bfk::BestRecord& best, uint32_t n, bf_result* out) {
+  std::memset(out, 0, sizeof *out);
+  if (best.ms >= 0xFFFFFFFFull) {
+    out->makespan_us = 0xFFFFFFFFu;
+    return;
+  }
+  out->index = best.idx;
+  out->makespan_us = (uint32_t)best.ms;
+  out->feasible = 1;
+  uint64_t idx = out->index;
+  for (uint32_t i = 0; i < n; ++i, idx /= 3) out->mode[i] = (uint8_t)(idx % 3);
 }
 
 }  // namespace bfcapi
@@ -402,6 +452,7 @@ int bf_create_scenario(const bf_scenario_desc* desc, bf_scenario** out) {
     whole_space_tables(s->tables, s->plan, s->window, split_and_window, &s->rtables, &s->rplan, &s->rwindow);
     split_and_window_pruned(s->rtables, &s->pplan, &s->pwindow);
   }
+  bfk::host::segment_plan(desc, makespan_bound(desc), &s->seg);
   cudaError_t e = cudaGetDevice(&s->device);
   bfk::LaneTreeRecord ltrec;
   if (e == cudaSuccess && desc->n >= bfk::kLtSingleMinTools && desc->n <= bfk::kLtMaxTools) {
@@ -422,7 +473,7 @@ int bf_create_scenario(const bf_scenario_desc* desc, bf_scenario** out) {
       s->lt_x = ltrec.x;
     }
   }
-  if (e == cudaSuccess) e = lib_malloc(reinterpret_cast<void**>(&s->d_scratch), sizeof(bf_scratch));
+  if (e == cudaSuccess) e = lib_malloc(reinterpret_cast<void**>(&s->d_scratch), kTableOffset + sizeof(uint32_t) * s->seg.entries);
   if (e == cudaSuccess) e = lib_malloc_host(reinterpret_cast<void**>(&s->h_scratch), sizeof(bf_scratch));
   if (e != cudaSuccess) {
     const int code = cuda_fail(e, "bf_create_scenario");
@@ -430,16 +481,18 @@ int bf_create_scenario(const bf_scenario_desc* desc, bf_scenario** out) {
     delete s;
     return code;
   }
+  s->d_table = reinterpret_cast<uint32_t*>(reinterpret_cast<unsigned char*>(s->d_scratch) + kTableOffset);
   s->d_key = &s->d_scratch->key;
   s->h_key = &s->h_scratch->key;
-  // The search kernel's launch state starts as (~0, 0, 0) and every launch
-  // leaves it so; its result goes to the pinned host mirror, which the
-  // device addresses directly.
+  // The launch states start as (~0, 0, ...) and every launch leaves them so;
+  // results go to the pinned host mirror, which the device addresses directly.
   void* mirror = nullptr;
-  e = cudaMemset(&s->d_scratch->search, 0, sizeof(bfk::SearchSync));
-  if (e == cudaSuccess) e = cudaMemset(&s->d_scratch->search.key, 0xFF, sizeof(unsigned long long));
-  if (e == cudaSuccess && s->lanetree)
-    e = cudaMemcpy(&s->d_scratch->lt, &ltrec, sizeof ltrec, cudaMemcpyHostToDevice);
+  bf_scratch::Launch& init = s->h_scratch->launch;
+  std::memset(&init, 0, sizeof init);
+  init.search.key = ~0ull;
+  std::memset(init.seg.key, 0xFF, sizeof init.seg.key);
+  if (s->lanetree) init.lt = ltrec;
+  e = cudaMemcpy(&s->d_scratch->launch, &init, sizeof init, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaHostGetDevicePointer(&mirror, s->h_scratch, 0);
   if (e != cudaSuccess) {
     const int code = cuda_fail(e, "bf_create_scenario");
@@ -448,7 +501,8 @@ int bf_create_scenario(const bf_scenario_desc* desc, bf_scenario** out) {
     delete s;
     return code;
   }
-  s->d_host_search_key = &static_cast<bf_scratch*>(mirror)->search.key;
+  s->d_host_search_key = &static_cast<bf_scratch*>(mirror)->launch.search.key;
+  s->d_host_best = &static_cast<bf_scratch*>(mirror)->best;
   *out = s;
   return BF_OK;
 }
@@ -477,8 +531,19 @@ int bf_eval_mappings(const bf_scenario* scn, uint64_t first, uint64_t count, uin
   if (count == 0) return BF_OK;
   if (!d_makespan || !d_feasible) return fail(BF_EINVAL, "bf_eval_mappings: NULL output buffer");
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  const bfk::Plan plan = make_plan(scn->plan, first, count, kSearchTasks);
   cudaError_t e = cudaSuccess;
+  // A captured launch may run after the handle is gone, so it takes the general
+  // kernel, whose tables travel by value.  Outside a capture the tables the
+  // sums read outlive the work: bf_destroy_scenario's cudaFree waits for it.
+  if (sums_pay(scn, count) && !is_capturing(st)) {
+    bfk::SegSums sums;
+    bfk::host::segment_sums(scn->seg, first, count, &sums);
+    e = bfk::launch_segment_tables(scn->seg, scn->d_table, st);
+    if (e == cudaSuccess) e = bfk::launch_segment_eval(sums, scn->d_table, d_makespan, d_feasible, st);
+    if (e != cudaSuccess) return cuda_fail(e, "bf_eval_mappings");
+    return BF_OK;
+  }
+  const bfk::Plan plan = make_plan(scn->plan, first, count, kSearchTasks);
 #define CALL(NW) launch_eval_nw##NW(scn->tables, scn->window, plan, d_makespan, d_feasible, st)
   BF_DISPATCH(bfk::bucket_for(scn->window.n), CALL)
 #undef CALL
@@ -618,6 +683,8 @@ int bf_search_pruned(const bf_scenario* scn_const, uint64_t hint_index, bf_resul
   const uint64_t total = pow3(n);
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   cudaError_t e = cudaSuccess;
+
+  if (scn->seg.count) return segment_optimum(scn, 3u, out, st, who);
 
   // 1. Incumbent: the best feasible of a few mappings (the hint, all-cpu,
   //    all-gpu_now, all-gpu_queue, each tool on its isolated-faster device).

@@ -11,13 +11,19 @@
 #include "bf_lanetree_launch.h"
 #include "bf_launch.h"
 #include "bf_plan.h"
+#include "bf_segments.h"
 #include "bf_tree.h"
 
 // Per-handle scratch, one block on the device and a pinned mirror on the host:
-// the packed search key, the tree search's best record, bound and counters,
-// the what-if probe list with its results, and the lane-tree record.
+// the launch states, the packed search key, the tree search's best record,
+// bound and counters, and the what-if probe list with its results.
 struct bf_scratch {
-  bfk::SearchSync search;  // whole-space searches' launch state; search.key of the host mirror receives their result
+  // Set at creation: what searches expect to find (and leave) in device memory.
+  struct Launch {
+    bfk::SearchSync search;  // whole-space searches; search.key of the host mirror receives their result
+    bfk::SegSync seg;        // branch and bound of scenarios cut by barriers
+    bfk::LaneTreeRecord lt;  // whole-space search by the lane-tree kernel (bf_scenario::lanetree)
+  } launch;
   unsigned long long key;
   uint32_t survivors;   // pruned search: number of surviving prefixes
   uint32_t pruned_bound;  // pruned search: the incumbent's makespan (set with survivors)
@@ -29,7 +35,6 @@ struct bf_scratch {
   uint64_t idx[BF_MAX_PROBES];
   uint32_t ms[BF_MAX_PROBES];
   uint8_t fe[BF_MAX_PROBES];
-  bfk::LaneTreeRecord lt;  // whole-space search by the lane-tree kernel (bf_scenario::lanetree)
 };
 
 struct bf_scenario {
@@ -51,12 +56,17 @@ struct bf_scenario {
   // and the blocks of a launch; lanetree false otherwise.
   bool lanetree;
   uint32_t lt_x, lt_blocks;
+  // Scenarios cut by barriers: the segments (seg.count = 0 otherwise), and
+  // their tables behind the device scratch, in the same allocation.
+  bfk::SegPlan seg;
+  uint32_t* d_table;
   int device;
   bf_scratch* d_scratch;      // device scratch
   bf_scratch* h_scratch;      // pinned host mirror
   unsigned long long* d_key;  // &d_scratch->key
   unsigned long long* h_key;  // &h_scratch->key
-  unsigned long long* d_host_search_key;  // &h_scratch->search.key as the device addresses it
+  unsigned long long* d_host_search_key;  // &h_scratch->launch.search.key as the device addresses it
+  bfk::BestRecord* d_host_best;           // &h_scratch->best as the device addresses it
   uint32_t* d_survivors;      // pruned search: 3^pplan.P prefix slots, allocated on first use
   uint32_t* d_levels;         // tree search: node buffers of every level, allocated on first use
   size_t levels_bytes;
@@ -77,6 +87,11 @@ int wait_stream(cudaStream_t st, const char* who);
 uint32_t wait_limit_ms();
 // BF_EINVAL unless the handle's device is current.
 int check_device(const bf_scenario* scn, const char* who);
+// The optimum of the full (radix 3) or binary space of a scenario cut by
+// barriers (scn->seg.count != 0), by one launch and one bounded wait.
+int segment_optimum(const bf_scenario* scn, uint32_t radix, bf_result* out, cudaStream_t st, const char* who);
+// A best record as a search's result.
+void fill_best(const volatile bfk::BestRecord& best, uint32_t n, bf_result* out);
 // Makespans of a list of mappings on the index-list kernel for the scenario's width.
 cudaError_t launch_list(const bf_scenario* scn, const uint64_t* idx, uint64_t count, uint32_t* ms, uint8_t* fe,
                         int grid, cudaStream_t st);

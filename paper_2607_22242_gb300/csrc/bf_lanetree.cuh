@@ -171,24 +171,22 @@ __device__ __forceinline__ void lt_fill_tables(LtSharedT<NC>& S) {
   }
   // Parts: root tools [0, min(x,4)), [4, min(x,8)), [8, min(x,12)), [12, x);
   // level tools [x, y), [y, n).
-  for (uint32_t p = 0; p < kLtParts; ++p) {
+  for (uint32_t e = threadIdx.x; e < kLtParts * kLtPartCombos; e += blockDim.x) {
+    const uint32_t p = e / kLtPartCombos, j = e - p * kLtPartCombos;
     const uint32_t lo = p < kLtRootParts ? min(kLtPartTools * p, R.x) : (p == kLtRootParts ? R.x : R.y);
     const uint32_t hi = p < kLtRootParts ? min(kLtPartTools * p + kLtPartTools, R.x) : (p == kLtRootParts ? R.y : R.n);
-    uint32_t combos = 1u;
-    for (uint32_t t = lo; t < hi; ++t) combos *= 3u;
-    for (uint32_t j = threadIdx.x; j < combos; j += blockDim.x) {
-      uint32_t now = 0u, que = 0u, idx = 0u, v = j;
-      for (uint32_t t = lo; t < hi; ++t) {
-        const uint32_t a = v % 3u;
-        v /= 3u;
-        now |= (a == 1u) ? (1u << t) : 0u;
-        que |= (a == 2u) ? (1u << t) : 0u;
-        idx += a * R.pv[t];
-      }
-      S.cnow[p][j] = now;
-      S.cque[p][j] = que;
-      S.cidx[p][j] = idx;
+    uint32_t now = 0u, que = 0u, idx = 0u, v = j;
+    for (uint32_t t = lo; t < hi; ++t) {
+      const uint32_t a = v % 3u;
+      v /= 3u;
+      now |= (a == 1u) ? (1u << t) : 0u;
+      que |= (a == 2u) ? (1u << t) : 0u;
+      idx += a * R.pv[t];
     }
+    if (v) continue;  // j is no combination of this part's tools
+    S.cnow[p][j] = now;
+    S.cque[p][j] = que;
+    S.cidx[p][j] = idx;
   }
   if (threadIdx.x == 0) {
     uint32_t* w = S.ck0;
@@ -202,7 +200,27 @@ __device__ __forceinline__ void lt_fill_tables(LtSharedT<NC>& S) {
   }
 }
 
-enum LtStep : uint32_t { kLtContinue = 0, kLtFinished = 1, kLtInfeasible = 2, kLtStopped = 3 };
+enum LtStep : uint32_t { kLtContinue = 0, kLtFinished = 1, kLtInfeasible = 2, kLtStopped = 3, kLtNoJob = 4 };
+
+// Modes and canonical index part of a root's tools: four table parts (base-81
+// digits of the root), of which a block skips those beyond its levels.
+template <uint32_t NC>
+__device__ __forceinline__ void lt_root_modes(const LtSharedT<NC>& S, uint32_t root, uint32_t* now, uint32_t* que,
+                                              uint32_t* idx) {
+  uint32_t q = root, n = 0u, w = 0u, x = 0u;
+#pragma unroll
+  for (uint32_t p = 0; p < kLtRootParts; ++p) {
+    if (p && kLtPartTools * p >= S.rec.x) break;
+    const uint32_t d = p + 1u < kLtRootParts ? q % kLtPartCombos : q;
+    q /= kLtPartCombos;
+    n |= S.cnow[p][d];
+    w |= S.cque[p][d];
+    x += S.cidx[p][d];
+  }
+  *now = n;
+  *que = w;
+  *idx = x;
+}
 
 // One step of a lane's simulation under modes (now, que; the other tools run
 // on the CPU): the admission at T -- or kLtStopped, before it, when a tool of
@@ -343,7 +361,8 @@ __device__ __forceinline__ uint32_t lt_step(const LtSharedT<NC>& S, LtState& s, 
 // which loads the block's time-0 state like a checkpoint -- and a stopped
 // job saves its state as the next level's checkpoint and continues with that
 // level's first combination (every tool of it on the CPU).
-template <uint32_t NC, bool W = false, typename TakeRoot, typename Sink>
+// DEAD: also report every infeasible mapping, through sink.dead(index).
+template <uint32_t NC, bool W = false, bool DEAD = false, typename TakeRoot, typename Sink>
 __device__ __forceinline__ void lt_lane(const LtSharedT<NC>& S, uint32_t* rows, uint32_t stride, TakeRoot take_root,
                                         Sink& sink) {
   constexpr uint32_t SW = lt_state_words<W>();
@@ -361,11 +380,20 @@ __device__ __forceinline__ void lt_lane(const LtSharedT<NC>& S, uint32_t* rows, 
   LtState s{};
   uint32_t now = 0u, que = 0u, stop = 0u, lvl = 0u, c1 = 0u, c2 = 0u;
   uint32_t idx0 = 0u, idx1 = 0u, idx2 = 0u, steps = 0u;
-  uint32_t r = kLtInfeasible;  // "the current job is over": the first pass takes a root
+  uint32_t r = kLtNoJob;  // the first pass takes a root
   for (;;) {
     if (r != kLtContinue) {
       // ---- the next job --------------------------------------------------
       if (r == kLtFinished) sink(idx0 + idx1 + idx2, s.T);
+      if constexpr (DEAD) {
+        if (r == kLtInfeasible) {  // every combination of the levels below the job's
+          const uint32_t below1 = lvl == 0u ? cnt1 : 1u, below2 = lvl <= 1u ? cnt2 : 1u;
+          for (uint32_t b = 0; b < below1; ++b)
+            for (uint32_t c = 0; c < below2; ++c)
+              sink.dead(idx0 + idx1 + idx2 + (lvl == 0u ? S.cidx[kLtRootParts][b] : 0u) +
+                        (lvl <= 1u ? S.cidx[kLtRootParts + 1u][c] : 0u));
+        }
+      }
       const bool descend = r == kLtStopped;
       const bool a2 = !descend && lvl == 2u && c2 + 1u < cnt2;
       const bool a1 = !descend && !a2 && lvl >= 1u && c1 + 1u < cnt1;
@@ -418,16 +446,7 @@ __device__ __forceinline__ void lt_lane(const LtSharedT<NC>& S, uint32_t* rows, 
       // first, all cpu, on a descent).
       uint32_t cn, cq, xi;
       if (L == 0u) {
-        uint32_t q = root;
-        cn = cq = xi = 0u;
-#pragma unroll
-        for (uint32_t p = 0; p < kLtRootParts; ++p) {
-          const uint32_t d = p + 1u < kLtRootParts ? q % kLtPartCombos : q;
-          q /= kLtPartCombos;
-          cn |= S.cnow[p][d];
-          cq |= S.cque[p][d];
-          xi += S.cidx[p][d];
-        }
+        lt_root_modes(S, root, &cn, &cq, &xi);
       } else {
         const uint32_t pa = L == 1u ? kLtRootParts : kLtRootParts + 1u, ia = L == 1u ? c1 : c2;
         cn = S.cnow[pa][ia];
