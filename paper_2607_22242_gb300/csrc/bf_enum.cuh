@@ -139,7 +139,7 @@ __device__ __forceinline__ void prefix_task(const TBF& tb, const SmemTables& sd,
     uint32_t r = kRunInfeasible;
     if ((dmid.que & tw.big_mask) == 0u) {
       load_lane(slotA, stride, w);
-      r = run<NW>(w, tw, sdw, rtw, dmid, inner_mask);
+      r = run<NW>(w, tw, sdw, rtw, dmid, inner_mask, plan.last_joins ? inner_mask : 0u);
     }
     if (plan.I == 0u) {  // no inner level: the run went to the end
       sink((uint32_t)base, r == kRunFinished ? w.T : kInfeasible);

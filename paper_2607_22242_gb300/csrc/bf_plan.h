@@ -254,8 +254,8 @@ inline void plan_for(const bfk::Tables& t, const uint32_t* anc, const uint32_t* 
   // lowers the compiled width (19-tool fan-out DAG: 8 -> 7 slots, 17.0 ->
   // 15.8 ms; at an unchanged width it measured 1 % slower).
   const uint32_t others = n >= 2 ? (1u << (n - 1)) - 1u : 0u;
-  pl->last_apart = (allow_apart && I == 1 && anc[n - 1] == others && n - w0 >= 2 &&
-                    bucket_for(n - w0 - 1) < bucket_for(n - w0))
+  pl->last_joins = I == 1 && anc[n - 1] == others ? 1u : 0u;
+  pl->last_apart = (allow_apart && pl->last_joins && n - w0 >= 2 && bucket_for(n - w0 - 1) < bucket_for(n - w0))
                        ? 1u
                        : 0u;
   std::memset(w, 0, sizeof *w);

@@ -343,7 +343,7 @@ __device__ __forceinline__ void leaf_combos(const TBW& tw, const SD& sdw, const 
       if (sim.que & tw.big_mask) continue;
       State<NW> w;
       load_lane(slot, stride, w);
-      if (run<NW>(w, tw, sdw, rtw, sim, 1u << lastw) != kRunStopped) continue;  // infeasible before it
+      if (run<NW>(w, tw, sdw, rtw, sim, 1u << lastw, 1u << lastw) != kRunStopped) continue;  // infeasible before it
       const Digits full{dg.now | (dc.now << W0), dg.que | (dc.que << W0)};
       for (uint32_t a = 0; a < tc.radix; ++a) {
         if (tc.alone[a] == kInfeasible) continue;
