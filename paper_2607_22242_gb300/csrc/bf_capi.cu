@@ -370,6 +370,15 @@ bool sums_pay(const bf_scenario* scn, uint64_t count) {
   return scn->seg.count != 0u && (scn->seg.tables == 0u || (count >= (1u << 17) && scn->seg.entries <= count / 2u));
 }
 
+// Whether a search of `count` mappings (not the whole space) of a scenario with
+// a lane-tree record runs on it: from an eighth of the space on.  Every root is
+// simulated whatever the range, so smaller ranges are the search kernel's
+// (its time, and the lane tree's, at 1/3, 1/9 and 1/27 of the space: 13-tool
+// sparse DAG 167, 87, 48 and 131, 113, 100 us; 14-tool layered DAG 429, 236, 83
+// and 262, 242, 234 us; 16-tool layered DAG 4.15, 3.21, 0.57 and 1.03, 0.83,
+// 0.69 ms; 18-tool layered DAG 17.5, 14.6, 4.9 and 4.2, 3.3, 3.1 ms).
+bool range_on_lanetree(const bf_scenario* scn, uint64_t count) { return count * 8u >= pow3(scn->desc.n); }
+
 // One launch of the search kernel -- or, for the whole space of a scenario
 // with a lane-tree record, of the lane-tree kernel; its last block writes
 // the best key into the host mirror (scn->h_scratch->search.key) and resets
@@ -383,9 +392,9 @@ int run_search(const bf_scenario* scn, uint64_t first, uint64_t count, bf_result
   // The whole space runs on the renumbered tables; a part of it keeps the
   // scenario's numbering, in which an index range is a box of the split.
   const bool whole = first == 0 && count == pow3(scn->desc.n);
-  if (whole && scn->lanetree) {
+  if (scn->lanetree && (whole || range_on_lanetree(scn, count))) {
     const cudaError_t e = bfk::launch_lanetree_single(&scn->d_scratch->launch.lt, scn->desc.n, scn->lt_x, scn->lt_blocks,
-                                                      &scn->d_scratch->launch.search, scn->d_host_search_key, st);
+                                                      (uint32_t)first, (uint32_t)(first + count - 1), &scn->d_scratch->launch.search, scn->d_host_search_key, st);
     if (e != cudaSuccess) return cuda_fail(e, who);
     const int rc = wait_stream(st, who);
     if (rc != BF_OK) return rc;

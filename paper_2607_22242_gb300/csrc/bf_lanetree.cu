@@ -84,11 +84,11 @@ __global__ void __launch_bounds__(kLtThreads, W ? kLtWideBlocksPerSm : kLtBlocks
 // finish copies it to *host_key (pinned host memory the device addresses)
 // and puts sync back to (~0, 0, 0).
 // NC table chunks, W the wide queue form: <3, false> up to 16 tools, <4,
-// true> up to 20.
-template <uint32_t NC, bool W>
+// true> up to 20.  RANGE: only canonical indices in [first, last].
+template <uint32_t NC, bool W, bool RANGE>
 __global__ void __launch_bounds__(kLtThreads, W ? kLtWideBlocksPerSm : kLtBlocksPerSm)
-    lanetree_single_kernel(const LaneTreeRecord* __restrict__ rec, uint32_t static_roots, SearchSync* sync,
-                           unsigned long long* host_key) {
+    lanetree_single_kernel(const LaneTreeRecord* __restrict__ rec, uint32_t static_roots, uint32_t first, uint32_t last,
+                           SearchSync* sync, unsigned long long* host_key) {
   extern __shared__ uint32_t lt_rows_smem[];
   __shared__ LtSharedT<NC> S;
   lt_load_record(S, rec);
@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(kLtThreads, W ? kLtWideBlocksPerSm : kLtBlocks
   for (uint32_t t = 0; t < S.rec.x; ++t) roots *= 3u;
   MinKeySink sink;
   LtSharedT<NC>& Sref = S;
-  lt_lane<NC, W>(S, lt_rows_smem + threadIdx.x, blockDim.x,
+  lt_lane<NC, W, false, RANGE>(S, lt_rows_smem + threadIdx.x, blockDim.x,
           [&Sref, sync, static_roots, roots]() {
             const uint32_t r = atomicAdd(&Sref.root_next, 1u);
             if (r < Sref.root_end) return r;
@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(kLtThreads, W ? kLtWideBlocksPerSm : kLtBlocks
             const uint32_t t = static_roots + base + __popc(group & ((1u << lane) - 1u));
             return t < roots ? t : 0xFFFFFFFFu;
           },
-          sink);
+          sink, first, last);
   const unsigned long long best = lt_warp_min(sink.best);
   if ((threadIdx.x & 31u) == 0u && best != ~0ull) atomicMin(&sync->key, best);
   __syncthreads();
@@ -134,17 +134,20 @@ size_t lt_smem_bytes(uint32_t n) { return sizeof(uint32_t) * lt_rows<W>(n) * kLt
 
 // The one-scenario kernel for n tools, with its dynamic shared memory allowed
 // (once per device and form).
-using SingleKernel = void (*)(const LaneTreeRecord*, uint32_t, SearchSync*, unsigned long long*);
-cudaError_t single_kernel_for(uint32_t n, SingleKernel* k, size_t* smem) {
-  static std::atomic<uint64_t> ready_narrow{0}, ready_wide{0};
-  if (n <= kLtNarrowTools) {
-    *k = lanetree_single_kernel<3, false>;
-    *smem = lt_smem_bytes<false>(n);
-    return allow_dyn_smem(lanetree_single_kernel<3, false>, lt_smem_bytes<false>(kLtNarrowTools), &ready_narrow);
-  }
-  *k = lanetree_single_kernel<4, true>;
-  *smem = lt_smem_bytes<true>(n);
-  return allow_dyn_smem(lanetree_single_kernel<4, true>, lt_smem_bytes<true>(kLtMaxTools), &ready_wide);
+using SingleKernel = void (*)(const LaneTreeRecord*, uint32_t, uint32_t, uint32_t, SearchSync*, unsigned long long*);
+template <uint32_t NC, bool W, bool RANGE>
+cudaError_t single_kernel_form(uint32_t n, uint32_t most, SingleKernel* k, size_t* smem) {
+  static std::atomic<uint64_t> ready{0};
+  *k = lanetree_single_kernel<NC, W, RANGE>;
+  *smem = lt_smem_bytes<W>(n);
+  return allow_dyn_smem(lanetree_single_kernel<NC, W, RANGE>, lt_smem_bytes<W>(most), &ready);
+}
+cudaError_t single_kernel_for(uint32_t n, bool range, SingleKernel* k, size_t* smem) {
+  if (n <= kLtNarrowTools)
+    return range ? single_kernel_form<3, false, true>(n, kLtNarrowTools, k, smem)
+                 : single_kernel_form<3, false, false>(n, kLtNarrowTools, k, smem);
+  return range ? single_kernel_form<4, true, true>(n, kLtMaxTools, k, smem)
+               : single_kernel_form<4, true, false>(n, kLtMaxTools, k, smem);
 }
 
 }  // namespace
@@ -176,7 +179,7 @@ cudaError_t launch_lanetree(const LaneTreeRecord* d_recs, const uint32_t* d_firs
 cudaError_t lanetree_single_blocks(uint32_t n, uint32_t* blocks) {
   SingleKernel k = nullptr;
   size_t smem = 0;
-  cudaError_t e = single_kernel_for(n, &k, &smem);
+  cudaError_t e = single_kernel_for(n, false, &k, &smem);
   int dev = 0, sms = 0, per_sm = 0;
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -187,15 +190,17 @@ cudaError_t lanetree_single_blocks(uint32_t n, uint32_t* blocks) {
 }
 
 cudaError_t launch_lanetree_single(const LaneTreeRecord* d_rec, uint32_t n, uint32_t x, uint32_t blocks,
-                                   SearchSync* sync, unsigned long long* host_key, cudaStream_t st) {
+                                   uint32_t first, uint32_t last, SearchSync* sync, unsigned long long* host_key,
+                                   cudaStream_t st) {
+  uint64_t roots = 1, total = 1;
+  for (uint32_t t = 0; t < x; ++t) roots *= 3u;
+  for (uint32_t t = 0; t < n; ++t) total *= 3u;
   SingleKernel k = nullptr;
   size_t smem = 0;
-  cudaError_t e = single_kernel_for(n, &k, &smem);
+  cudaError_t e = single_kernel_for(n, first != 0u || last + 1u != total, &k, &smem);
   if (e != cudaSuccess) return e;
-  uint64_t roots = 1;
-  for (uint32_t t = 0; t < x; ++t) roots *= 3u;
   const uint32_t static_roots = (uint32_t)(roots * kLtStaticShareNum / kLtStaticShareDen);
-  k<<<blocks, kLtThreads, smem, st>>>(d_rec, static_roots, sync, host_key);
+  k<<<blocks, kLtThreads, smem, st>>>(d_rec, static_roots, first, last, sync, host_key);
   return cudaGetLastError();
 }
 

@@ -362,9 +362,13 @@ __device__ __forceinline__ uint32_t lt_step(const LtSharedT<NC>& S, LtState& s, 
 // job saves its state as the next level's checkpoint and continues with that
 // level's first combination (every tool of it on the CPU).
 // DEAD: also report every infeasible mapping, through sink.dead(index).
-template <uint32_t NC, bool W = false, bool DEAD = false, typename TakeRoot, typename Sink>
+// RANGE: only mappings with canonical indices in [first, last] are simulated to
+// the end and reported; a root or a combination none of whose mappings can lie
+// in the range (between its own index part and that plus twice the open tools'
+// place values) is passed over.
+template <uint32_t NC, bool W = false, bool DEAD = false, bool RANGE = false, typename TakeRoot, typename Sink>
 __device__ __forceinline__ void lt_lane(const LtSharedT<NC>& S, uint32_t* rows, uint32_t stride, TakeRoot take_root,
-                                        Sink& sink) {
+                                        Sink& sink, uint32_t first = 0u, uint32_t last = 0xFFFFFFFFu) {
   constexpr uint32_t SW = lt_state_words<W>();
   const LaneTreeRecord& R = S.rec;
   const uint32_t n = R.n;
@@ -376,6 +380,14 @@ __device__ __forceinline__ void lt_lane(const LtSharedT<NC>& S, uint32_t* rows, 
   for (uint32_t t = R.x; t < R.y; ++t) cnt1 *= 3u;
   for (uint32_t t = R.y; t < n; ++t) cnt2 *= 3u;
   const uint32_t bound = n + 2u;  // steps of one job: each event retires a tool
+  uint32_t open1 = 0u, open2 = 0u;  // RANGE: the largest index part of the tools below a root, of level 2
+  if constexpr (RANGE) {
+    for (uint32_t t = R.x; t < n; ++t) open1 += 2u * R.pv[t];
+    for (uint32_t t = R.y; t < n; ++t) open2 += 2u * R.pv[t];
+  }
+  auto overlaps = [&](uint32_t idx, uint32_t open) {
+    return !RANGE || (idx <= last && (uint64_t)idx + open >= first);
+  };
 
   LtState s{};
   uint32_t now = 0u, que = 0u, stop = 0u, lvl = 0u, c1 = 0u, c2 = 0u;
@@ -394,16 +406,38 @@ __device__ __forceinline__ void lt_lane(const LtSharedT<NC>& S, uint32_t* rows, 
                         (lvl <= 1u ? S.cidx[kLtRootParts + 1u][c] : 0u));
         }
       }
-      const bool descend = r == kLtStopped;
-      const bool a2 = !descend && lvl == 2u && c2 + 1u < cnt2;
-      const bool a1 = !descend && !a2 && lvl >= 1u && c1 + 1u < cnt1;
-      const uint32_t L = descend ? lvl + 1u : (a2 ? 2u : (a1 ? 1u : 0u));
-      c1 = (descend && L == 1u) ? 0u : (a1 ? c1 + 1u : c1);
-      c2 = (descend && L == 2u) ? 0u : (a2 ? c2 + 1u : c2);
-      uint32_t root = 0u;
+      // A stopped job descends to its first combination of the next level,
+      // saving its state; else the next combination of the deepest level that
+      // has one left resumes that level's checkpoint, or a new root starts.
+      bool descend = r == kLtStopped;
+      uint32_t L;
+      if constexpr (RANGE) {
+        L = r == kLtNoJob ? 0u : (descend ? lvl + 1u : lvl);
+        if (L == 2u) {
+          c2 = descend ? 0u : c2 + 1u;
+          while (c2 < cnt2 && !overlaps(idx0 + idx1 + S.cidx[kLtRootParts + 1u][c2], 0u)) ++c2;
+          if (c2 >= cnt2) L = 1u;
+        }
+        if (L == 1u) {
+          c1 = descend && lvl == 0u ? 0u : c1 + 1u;
+          while (c1 < cnt1 && !overlaps(idx0 + S.cidx[kLtRootParts][c1], open2)) ++c1;
+          if (c1 >= cnt1) L = 0u;
+        }
+        descend = descend && L == lvl + 1u;
+      } else {
+        const bool a2 = !descend && lvl == 2u && c2 + 1u < cnt2;
+        const bool a1 = !descend && !a2 && lvl >= 1u && c1 + 1u < cnt1;
+        L = descend ? lvl + 1u : (a2 ? 2u : (a1 ? 1u : 0u));
+        c1 = (descend && L == 1u) ? 0u : (a1 ? c1 + 1u : c1);
+        c2 = (descend && L == 2u) ? 0u : (a2 ? c2 + 1u : c2);
+      }
+      uint32_t root = 0u, cn, cq, xi;
       if (L == 0u) {
-        root = take_root();
-        if (root == 0xFFFFFFFFu) return;
+        do {
+          root = take_root();
+          if (root == 0xFFFFFFFFu) return;
+          if constexpr (RANGE) lt_root_modes(S, root, &cn, &cq, &xi);
+        } while (RANGE && !overlaps(xi, open1));
       }
       uint32_t* const cw = rows + (L == 2u ? n + SW : n) * stride;  // checkpoint L's state words
       if (descend) {  // save the state words
@@ -441,12 +475,10 @@ __device__ __forceinline__ void lt_lane(const LtSharedT<NC>& S, uint32_t* rows, 
           s.qhi = (uint64_t)w[10u * ws] | ((uint64_t)w[11u * ws] << 32);
         }
       }
-      // Modes and index part of the new job's level: a root's four table
-      // parts (base-81 digits of the root), or one level combination (the
-      // first, all cpu, on a descent).
-      uint32_t cn, cq, xi;
+      // Modes and index part of the new job's level: a root's, or one level
+      // combination (the first on a descent).
       if (L == 0u) {
-        lt_root_modes(S, root, &cn, &cq, &xi);
+        if constexpr (!RANGE) lt_root_modes(S, root, &cn, &cq, &xi);
       } else {
         const uint32_t pa = L == 1u ? kLtRootParts : kLtRootParts + 1u, ia = L == 1u ? c1 : c2;
         cn = S.cnow[pa][ia];

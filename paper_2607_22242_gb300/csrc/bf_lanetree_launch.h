@@ -35,10 +35,12 @@ constexpr uint64_t kLtStaticShareNum = 1, kLtStaticShareDen = 2;
 // resident slot of every SM.
 cudaError_t lanetree_single_blocks(uint32_t n, uint32_t* blocks);
 
-// One launch over d_rec (n tools, roots [0, 3^x)); *sync must hold (~0, 0, 0)
+// One launch over the mappings of d_rec (n tools, roots [0, 3^x)) with
+// canonical indices in [first, last]; *sync must hold (~0, 0, 0)
 // and is left so; the lowest key (makespan << 32 | canonical index, ~0 when
 // no mapping is feasible) is written to *host_key by the last block.
 cudaError_t launch_lanetree_single(const LaneTreeRecord* d_rec, uint32_t n, uint32_t x, uint32_t blocks,
-                                   SearchSync* sync, unsigned long long* host_key, cudaStream_t st);
+                                   uint32_t first, uint32_t last, SearchSync* sync, unsigned long long* host_key,
+                                   cudaStream_t st);
 
 }  // namespace bfk
