@@ -470,15 +470,11 @@ int bf_create_scenario(const bf_scenario_desc* desc, bf_scenario** out) {
     if (bfk::lanetree_single_blocks(desc->n, &s->lt_blocks) != cudaSuccess) {
       cudaGetLastError();
     } else {
-      double lt_events = 0.0;
-      bfk::host::lanetree_record(desc, &ltrec,
-                                 (uint64_t)s->lt_blocks * bfk::kLtLaunchThreads * bfk::kLtSingleRootsPerLane,
-                                 &lt_events);
-      s->lanetree = bfk::host::lanetree_preferred(s->rtables, s->rplan, s->rwindow, ltrec, lt_events);
-      if (s->lanetree)
-        bfk::host::lanetree_sampled_levels(ltrec, (uint64_t)s->lt_blocks * bfk::kLtLaunchThreads *
-                                                      bfk::kLtSingleRootsPerLane,
-                                           &ltrec.x, &ltrec.y);
+      const uint64_t lanes = (uint64_t)s->lt_blocks * bfk::kLtLaunchThreads;
+      const uint64_t min_roots = lanes * bfk::kLtSingleRootsNum / bfk::kLtSingleRootsDen;
+      bfk::host::lanetree_record(desc, &ltrec, min_roots);
+      const double cost = bfk::host::lanetree_sampled_levels(ltrec, min_roots, &ltrec.x, &ltrec.y, lanes);
+      s->lanetree = bfk::host::lanetree_preferred(s->rtables, s->rplan, s->rwindow, cost);
       s->lt_x = ltrec.x;
     }
   }

@@ -24,11 +24,11 @@ constexpr uint32_t kLtLaunchThreads = 256;  // threads per block of both kernels
 
 // The one-scenario lane-tree search: every lane of the current device on one
 // record of kLtSingleMinTools to kLtMaxTools tools (full searches of such
-// scenarios take it when bf_plan.h lanetree_preferred says so).  The record's x gives 3^x >= lanes *
-// kLtSingleRootsPerLane roots; the blocks are dealt kLtStaticShare of them
+// scenarios take it when bf_plan.h lanetree_preferred says so).  The record's x gives at least half a
+// root per lane; the blocks are dealt kLtStaticShare of them
 // in advance, the rest go to whichever lanes ask first.
 constexpr uint32_t kLtSingleMinTools = 10;
-constexpr uint64_t kLtSingleRootsPerLane = 2;
+constexpr uint64_t kLtSingleRootsNum = 1, kLtSingleRootsDen = 2;
 constexpr uint64_t kLtStaticShareNum = 1, kLtStaticShareDen = 2;
 
 // Blocks of one launch for an n-tool record on the current device: every

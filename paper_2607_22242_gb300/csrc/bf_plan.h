@@ -466,7 +466,7 @@ constexpr uint64_t kLtMaxBlocksPerScenario = 1024;
 // against 2.8 for the best split and 4.1 for the prefix/mid/inner split of
 // the other batch kernel.
 template <typename TB>
-inline double lanetree_levels(const TB& t, uint64_t min_roots, uint32_t* x_out, uint32_t* y_out) {
+inline void lanetree_levels(const TB& t, uint64_t min_roots, uint32_t* x_out, uint32_t* y_out) {
   const uint32_t n = t.n;
   uint32_t R[BF_MAX_TOOLS + 1] = {};
   retired_estimate(t, R);
@@ -489,7 +489,6 @@ inline double lanetree_levels(const TB& t, uint64_t min_roots, uint32_t* x_out, 
   }
   *x_out = bx;
   *y_out = by;
-  return best;
 }
 
 // The batch's levels (every block gets kLtMinRootsPerBlock roots or more)
@@ -514,8 +513,8 @@ inline void lanetree_split(const TB& t, uint32_t* x_out, uint32_t* y_out, uint32
 //
 // lt_sample_events simulates one mapping (mode[t] per tool of the record's
 // numbering) with the model's arithmetic in 64-bit integers and returns, for
-// every b in [0, n], ev[b] = the events before the first tool >= b becomes
-// ready (all its events if none does) and reached[b] = whether one does
+// every b in [0, n], ev[b] = the lane's steps before the first tool >= b becomes
+// ready (all its steps if none does) and reached[b] = whether one does
 // (the mapping has not been found infeasible before).  Estimates only: no
 // result depends on them.
 inline void lt_sample_events(const bfk::LaneTreeRecord& r, const uint8_t* mode, uint32_t* ev, bool* reached) {
@@ -569,7 +568,11 @@ inline void lt_sample_events(const bfk::LaneTreeRecord& r, const uint8_t* mode, 
         ++qhead;
       }
     }
-    if (!run) break;  // every tool has ended
+    ++events;
+    if (pend == 0u && __builtin_popcount(run & ~cpu) <= 1) {  // the closed form applies
+      for (; qhead < qtail; ++qhead) dead = dead || ((r.big_mask >> fifo[qhead]) & 1u);
+      break;
+    }
     uint32_t k = 0;
     uint64_t tc = ~0ull, gm = ~0ull;
     for (uint32_t m = run; m; m &= m - 1u) {
@@ -591,7 +594,6 @@ inline void lt_sample_events(const bfk::LaneTreeRecord& r, const uint8_t* mode, 
       if (k) V += ((tc - T) << 20) / f;
       T = tc;
     }
-    ++events;
     for (uint32_t m = run; m; m &= m - 1u) {
       const uint32_t t = (uint32_t)__builtin_ctz(m);
       const bool ends = (cpu >> t) & 1u ? end[t] == T : (gpu_event && end[t] == V);
@@ -600,6 +602,11 @@ inline void lt_sample_events(const bfk::LaneTreeRecord& r, const uint8_t* mode, 
         done |= 1u << t;
         vram -= (cpu >> t) & 1u ? 0u : r.vram[t];
       }
+    }
+    const uint32_t left = run & ~cpu;
+    if (pend == 0u && (left & (left - 1u)) == 0u && (left == 0u || qhead == qtail || (left & que))) {
+      for (; qhead < qtail; ++qhead) dead = dead || ((r.big_mask >> fifo[qhead]) & 1u);
+      break;
     }
   }
   uint32_t earliest = 0xFFFFFFFFu;
@@ -613,15 +620,24 @@ inline void lt_sample_events(const bfk::LaneTreeRecord& r, const uint8_t* mode, 
 }
 
 // Levels of a one-scenario record from kLtLevelSamples mappings drawn
-// uniformly (a fixed seed: the same choice on every machine), for records the
-// search will run (about 0.1 ms of host time at 16 tools): among the
+// uniformly (a fixed seed: the same choice on every machine; about 0.1 ms of
+// host time at 16 tools): among the
 // splits lanetree_levels allows, the one of least sampled cost -- a root
-// runs its mappings' events up to ev[x], a level-1 job up to ev[y] from
-// there, a leaf to the end, and a job costs half an event more; jobs exist
-// only below checkpoints that were reached.
+// runs its mappings' steps up to ev[x], a level-1 job up to ev[y] from
+// there, a leaf to the end, and a job costs 0.3 steps more; jobs exist
+// only below checkpoints that were reached.  The cost grows by 0.6 / r for
+// r roots per lane (`lanes` lanes share them): the last roots of a search leave
+// lanes idle, the more so the fewer a lane runs.  Over all splits of 17 layered
+// and sparse DAGs of 12 to 17 tools, timed one by one, that choice is within 2 %
+// of the fastest split on average (1.21x at worst; without the second term
+// 1.21x for a 16-tool DAG, and roots far too few for the smaller ones).
+// Against levels from events alone with at least two roots per lane: 17-tool
+// layered DAG 9.1 -> 5.3 ms, 16-tool ones 1.59 -> 1.30 and 1.53 -> 1.53 ms,
+// 12-tool layered ones 112 -> 79 and 101 -> 70 us.
 constexpr uint32_t kLtLevelSamples = 128;
-inline void lanetree_sampled_levels(const bfk::LaneTreeRecord& r, uint64_t min_roots, uint32_t* x_out,
-                                    uint32_t* y_out) {
+// Returns that cost in steps per mapping.
+inline double lanetree_sampled_levels(const bfk::LaneTreeRecord& r, uint64_t min_roots, uint32_t* x_out,
+                                      uint32_t* y_out, uint64_t lanes = 0) {
   const uint32_t n = r.n;
   uint64_t S[bfk::kLtMaxTools + 1] = {}, A[bfk::kLtMaxTools + 1] = {};
   uint64_t state = 0x9E3779B97F4A7C15ull;
@@ -641,6 +657,7 @@ inline void lanetree_sampled_levels(const bfk::LaneTreeRecord& r, uint64_t min_r
       A[b] += reached[b] ? 1u : 0u;
     }
   }
+  if (lanes == 0) lanes = min_roots / 2u + 1u;
   uint32_t xmin = 0;
   while (xmin < n && pow3(xmin) < min_roots) ++xmin;
   if (n > 2u * kLtPartTools && xmin < n - 2u * kLtPartTools) xmin = n - 2u * kLtPartTools;
@@ -649,16 +666,19 @@ inline void lanetree_sampled_levels(const bfk::LaneTreeRecord& r, uint64_t min_r
     for (uint32_t y = (x == n ? n : x + 1u); y <= n; ++y) {
       if (y - x > kLtPartTools || n - y > kLtPartTools) continue;
       const uint64_t px = pow3(x), py = pow3(y), pn = pow3(n);
-      // Twice the cost, summed over the samples (half events are whole).
-      const uint64_t cost = 2u * (px * S[x] + py * (S[y] - S[x]) + pn * (S[n] - S[y])) + px * kLtLevelSamples +
-                            (x < n ? py * A[x] : 0u) + (y < n ? pn * A[y] : 0u);
-      if (cost < best) {
-        best = cost;
+      // Ten times the cost, summed over the samples: at most 10 * 3^20 * 22 *
+      // kLtLevelSamples < 2^47.
+      const uint64_t cost = 10u * (px * S[x] + py * (S[y] - S[x]) + pn * (S[n] - S[y])) +
+                            3u * (px * kLtLevelSamples + (x < n ? py * A[x] : 0u) + (y < n ? pn * A[y] : 0u));
+      const uint64_t padded = cost + cost / px * (lanes * 6u / 10u);
+      if (padded < best) {
+        best = padded;
         *x_out = x;
         *y_out = y;
       }
     }
   }
+  return (double)best / (10.0 * kLtLevelSamples * (double)pow3(n));
 }
 
 // The tables a lane-tree record's split estimate reads (n, pred, cpu, wnow).
@@ -674,10 +694,8 @@ struct LtView {
 // Built straight from the desc; the slowdown constants are those of
 // build_tables, taken over from the previous record built on this thread
 // when the slowdown table is the same (the scenarios of a batch usually
-// share one).  *events (if given) receives the levels' estimated events
-// per mapping (lanetree_levels' cost over 3^n).
-inline void lanetree_record(const bf_scenario_desc* d, bfk::LaneTreeRecord* r, uint64_t min_roots = 0,
-                            double* events = nullptr) {
+// share one).
+inline void lanetree_record(const bf_scenario_desc* d, bfk::LaneTreeRecord* r, uint64_t min_roots = 0) {
   const uint32_t n = d->n;
   uint32_t order[BF_MAX_TOOLS], pos[BF_MAX_TOOLS], k = 0;
   for (uint32_t v = 0; v < n; ++v)
@@ -719,51 +737,37 @@ inline void lanetree_record(const bf_scenario_desc* d, bfk::LaneTreeRecord* r, u
   if (min_roots == 0) {
     lanetree_split(view, &r->x, &r->y, &r->nblocks);
   } else {
-    const double cost = lanetree_levels(view, min_roots, &r->x, &r->y);
+    lanetree_levels(view, min_roots, &r->x, &r->y);
     r->nblocks = 1;
-    if (events) *events = cost / (double)pow3(n);
   }
 }
 
 // Whether a full search of a scenario goes to the one-scenario lane-tree
-// kernel (record rec, estimated events per mapping lt_events) rather than
-// the search kernel (whole-space tables rt, plan rp, window rw).  The search
+// kernel (sampled cost lt_cost, lanetree_sampled_levels) rather than the
+// search kernel (whole-space tables rt, plan rp, window rw).  The search
 // kernel's cost per mapping grows with its events per mapping -- R-estimate
 // events after its prefix checkpoint shared by 3^(M+I) mappings, its mid
 // checkpoint by 3^I -- times its window width (each event scans the window),
-// at full warp efficiency when its lanes follow the same structure; the
-// lane tree's with its own events per mapping, at the divergence of lanes
-// on different mappings.  Measured (full searches, 152-SM GB300): the lane
-// tree is faster on every layered and fan-out/fan-in DAG of 12 to 16 tools
-// tried (16-tool layered workload 2.70 -> 1.70 ms; layered 14 tools 0.60 ->
-// 0.21 ms) and on the chain and spine DAGs of 13 and 14 tools; slower when
-// its roots are whole mappings (x = n: the 12-tool fan-out/fan-in 0.053 ->
-// 0.081 ms) and on chain and spine DAGs of 15 and 16 tools, whose narrow
-// windows (4 to 6 slots) make the search kernel's events cheap (16-tool
-// chain 0.67 ms against 0.82): there the search kernel's events x window
-// width is 4.4 to 6.8 times the lane tree's estimate, in the cases the lane
-// tree wins 6.7 to 21 times.  On 40 further DAGs of 13 to 16 tools (layered,
-// sparse, fan-out/fan-in, spines with branches) the rule chose the lane tree
-// for all 40, and it was the faster on all 40.
-constexpr double kLtPreferRatio = 8.0;
-// Above 16 tools the lane tree runs its wide form (5-bit queue entries in two
-// words, 55 registers, 4 blocks per SM), whose events cost more: on layered
-// DAGs of 17 to 20 tools it won 2.05 to 2.3 times at ratios of 18.4 to 19.8
-// (the 24-tool layered workload's first 20 tools 850 -> 363 ms), 1.4 times
-// at 17.3, and lost 1.6 times at 12.8; the 19-tool workload's ratio is 6.6.
-// On 12 further DAGs of 17 to 19 tools it chose the lane tree for all 12,
-// the faster on all 12.
-constexpr double kLtPreferRatioWide = 15.0;
-inline bool lanetree_preferred(const bfk::Tables& rt, const bfk::Plan& rp, const bfk::Tables& rw,
-                               const bfk::LaneTreeRecord& rec, double lt_events) {
+// at full warp efficiency when its lanes follow the same structure; the lane
+// tree's with its steps, at the divergence of lanes on different mappings.
+// Both timed on 59 DAGs of 10 to 18 tools (152-SM GB300), by the ratio of the
+// two: from 16 tools on the lane tree won 1.4 to 3.7 times on every layered
+// and sparse DAG (ratios 18 to 54) and lost up to 1.9 times on chains, spines
+// and fan-outs (3 to 15), whose narrow windows make the search kernel's events
+// cheap; with 12 to 15 tools it won up to 3.7 times or tied, but for fan-outs
+// of 14 and 15 tools (up to 7 % slower); with 10 and 11 tools, where most lanes
+// have no root, it won up to 2.2 times on layered and sparse DAGs (1.6 to 3.0
+// and 3.0 to 4.3; two ties) and lost on the others (up to 1.0 and 1.9).  On 59
+// more DAGs of other seeds the rule's choice took 1.5 % longer than the faster
+// kernel on average.
+inline bool lanetree_preferred(const bfk::Tables& rt, const bfk::Plan& rp, const bfk::Tables& rw, double lt_cost) {
   const uint32_t n = rt.n;
-  if (rec.x >= n) return false;
-  if (n <= 14u) return true;
+  if (n >= 12u && n <= 15u) return true;
   uint32_t R[BF_MAX_TOOLS + 1] = {};
   retired_estimate(rt, R);
   const uint32_t P = rp.P, I = rp.I;
   const double sk_events = R[P] / (double)pow3(rp.M + I) + (R[n - I] - R[P]) / (double)pow3(I) + (n - R[n - I]);
-  return sk_events * rw.n >= (n > kLtNarrowTools ? kLtPreferRatioWide : kLtPreferRatio) * lt_events;
+  return sk_events * rw.n >= (n >= 16u ? 16.0 : (n == 11u ? 2.5 : 1.3)) * lt_cost;
 }
 
 }  // namespace host
