@@ -94,6 +94,97 @@ uint64_t makespan_bound(const bf_scenario_desc* d) {
   return bound;
 }
 
+// The driver's cuCtxGetCurrent and cuCtxGetId, looked up through the runtime
+// (the library links no driver library).
+using CtxGetCurrentFn = CUresult (*)(CUcontext*);
+using CtxGetIdFn = CUresult (*)(CUcontext, unsigned long long*);
+struct CtxFns {
+  CtxGetCurrentFn get_current = nullptr;
+  CtxGetIdFn get_id = nullptr;
+};
+
+const CtxFns& ctx_fns() {
+  static const CtxFns fns = [] {
+    CtxFns f;
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      f.get_current = reinterpret_cast<CtxGetCurrentFn>(p);
+    p = nullptr;
+    if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      f.get_id = reinterpret_cast<CtxGetIdFn>(p);
+    return f;
+  }();
+  return fns;
+}
+
+// ID of the current context, 0 when none is current yet.
+int current_ctx_id(unsigned long long* id, const char* who) {
+  const CtxFns& f = ctx_fns();
+  if (!f.get_current || !f.get_id) return fail(BF_ECUDA, "%s: cuCtxGetCurrent/cuCtxGetId not available", who);
+  CUcontext ctx = nullptr;
+  if (f.get_current(&ctx) != CUDA_SUCCESS) return fail(BF_ECUDA, "%s: cuCtxGetCurrent failed", who);
+  *id = 0;
+  if (ctx && f.get_id(ctx, id) != CUDA_SUCCESS) return fail(BF_ECUDA, "%s: cuCtxGetId failed", who);
+  return BF_OK;
+}
+
+// Scratch of handles that are gone (a device block and its pinned mirror, 14 KB
+// each), for the next handles: allocating and freeing them took most of a
+// one-off search (12-tool fan-out through bf_create_scenario, bf_search_best
+// and bf_destroy_scenario: 547 -> 118 us).  At most kMost pairs are kept; a pair
+// belongs to the context it was made in and is only handed out there.
+class ScratchPool {
+ public:
+  struct Pair {
+    bf_scratch* d;
+    bf_scratch* h;
+  };
+
+  // A pair made in the current context, or false.
+  bool take(Pair* out) {
+    unsigned long long id = 0;
+    if (!context(&id)) return false;
+    std::lock_guard<std::mutex> lock(mu_);
+    for (unsigned i = 0; i < count_; ++i)
+      if (slots_[i].ctx == id) {
+        *out = slots_[i].pair;
+        slots_[i] = slots_[--count_];
+        return true;
+      }
+    return false;
+  }
+
+  // Keep a pair of the current context; false (the caller frees it) when the
+  // pool is full or the context cannot be told.
+  bool keep(const Pair& pair) {
+    unsigned long long id = 0;
+    if (!context(&id)) return false;
+    std::lock_guard<std::mutex> lock(mu_);
+    if (count_ == kMost) return false;
+    slots_[count_++] = Slot{id, pair};
+    return true;
+  }
+
+ private:
+  static constexpr unsigned kMost = 16;
+  struct Slot {
+    unsigned long long ctx;
+    Pair pair;
+  };
+  static bool context(unsigned long long* id) {
+    const CtxFns& f = ctx_fns();
+    CUcontext ctx = nullptr;
+    return f.get_current && f.get_id && f.get_current(&ctx) == CUDA_SUCCESS && ctx && f.get_id(ctx, id) == CUDA_SUCCESS;
+  }
+  std::mutex mu_;
+  Slot slots_[kMost];
+  unsigned count_ = 0;
+};
+ScratchPool g_scratch_pool;
+
 int validate(const bf_scenario_desc* d, const char* who) {
   if (!d) return fail(BF_EINVAL, "%s: desc is NULL", who);
   const uint32_t n = d->n;
@@ -140,6 +231,14 @@ int wait_stream(cudaStream_t st, const char* who) {
     // millisecond or two.  Longer waits sleep 20 us between polls.
     if (us > 5000) std::this_thread::sleep_for(std::chrono::microseconds(20));
   }
+}
+
+void begin_call(const bf_scenario* scn) { const_cast<bf_scenario*>(scn)->busy = true; }
+
+int end_call(const bf_scenario* scn, cudaStream_t st, const char* who) {
+  const int rc = wait_stream(st, who);
+  if (rc == BF_OK) const_cast<bf_scenario*>(scn)->busy = false;
+  return rc;
 }
 
 // A handle's scratch lives on the device that was current at creation; its
@@ -333,20 +432,11 @@ void build_lanetree_records(const bf_scenario_desc* descs, const uint32_t* ids, 
   });
 }
 
-constexpr size_t align256(size_t x) { return (x + 255) / 256 * 256; }
-constexpr size_t kTableOffset = align256(sizeof(bf_scratch));  // the segments' tables, behind the scratch
+inline size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
-// Index-list evaluation: the 20-slot kernels up to 20 tools, the 32-slot one above.
 cudaError_t launch_list(const bf_scenario* scn, const uint64_t* idx, uint64_t count, uint32_t* ms, uint8_t* fe,
-                        int grid, cudaStream_t st) {
-  const uint32_t n = scn->desc.n;
-  const uint64_t total = pow3(n);
-  if (n > BF_MAX_TOOLS_ENUM) return bfk::launch_wide_list(scn->wide, total, idx, count, ms, fe, grid, st);
-  cudaError_t e = cudaSuccess;
-#define CALL(NW) launch_list_nw##NW(scn->tables, total, idx, count, ms, fe, grid, st)
-  BF_DISPATCH(bfk::bucket_for(n), CALL)
-#undef CALL
-  return e;
+                        cudaStream_t st) {
+  return bfk::launch_lanetree_list(scn->wide, pow3(scn->desc.n), idx, count, ms, fe, st);
 }
 
 // Whether work put on `st` is being captured (or whether that cannot be told).
@@ -368,6 +458,23 @@ bool is_capturing(cudaStream_t st) {
 // 50 us; 2^25 mappings of the 19-tool spine 47 us against 1.57 ms).
 bool sums_pay(const bf_scenario* scn, uint64_t count) {
   return scn->seg.count != 0u && (scn->seg.tables == 0u || (count >= (1u << 17) && scn->seg.entries <= count / 2u));
+}
+
+// The memory of the segments' tables, allocated by the handle's first evaluation
+// that uses them (threads may evaluate on one handle at once: the first pointer
+// stored stays); false if it cannot be had, and the general kernel runs.
+bool segment_tables(const bf_scenario* scn, uint32_t** table) {
+  uint32_t** slot = const_cast<uint32_t**>(&scn->d_table);
+  *table = __atomic_load_n(slot, __ATOMIC_ACQUIRE);
+  if (*table || scn->seg.entries == 0u) return true;
+  uint32_t* mine = nullptr;
+  if (lib_malloc(reinterpret_cast<void**>(&mine), sizeof(uint32_t) * scn->seg.entries) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  if (__atomic_compare_exchange_n(slot, table, mine, false, __ATOMIC_ACQ_REL, __ATOMIC_ACQUIRE)) *table = mine;
+  else cudaFree(mine);
+  return true;
 }
 
 // Whether a search of `count` mappings (not the whole space) of a scenario with
@@ -392,11 +499,12 @@ int run_search(const bf_scenario* scn, uint64_t first, uint64_t count, bf_result
   // The whole space runs on the renumbered tables; a part of it keeps the
   // scenario's numbering, in which an index range is a box of the split.
   const bool whole = first == 0 && count == pow3(scn->desc.n);
+  begin_call(scn);
   if (scn->lanetree && (whole || range_on_lanetree(scn, count))) {
     const cudaError_t e = bfk::launch_lanetree_single(&scn->d_scratch->launch.lt, scn->desc.n, scn->lt_x, scn->lt_blocks,
-                                                      (uint32_t)first, (uint32_t)(first + count - 1), &scn->d_scratch->launch.search, scn->d_host_search_key, st);
+                                                      (uint32_t)first, (uint32_t)(first + count - 1), &scn->d_scratch->launch.search, &scn->d_host_scratch->launch.search.key, st);
     if (e != cudaSuccess) return cuda_fail(e, who);
-    const int rc = wait_stream(st, who);
+    const int rc = end_call(scn, st, who);
     if (rc != BF_OK) return rc;
     fill_result(*static_cast<volatile unsigned long long*>(&scn->h_scratch->launch.search.key), scn->desc.n, first, out);
     return BF_OK;
@@ -405,21 +513,22 @@ int run_search(const bf_scenario* scn, uint64_t first, uint64_t count, bf_result
   const bfk::Tables& tw = whole ? scn->rwindow : scn->window;
   const bfk::Plan plan = make_plan(whole ? scn->rplan : scn->plan, first, count, kSearchTasks);
   cudaError_t e = cudaSuccess;
-#define CALL(NW) launch_search_nw##NW(tb, tw, plan, &scn->d_scratch->launch.search, scn->d_host_search_key, st)
+#define CALL(NW) launch_search_nw##NW(tb, tw, plan, &scn->d_scratch->launch.search, &scn->d_host_scratch->launch.search.key, st)
   BF_DISPATCH(bfk::bucket_for(tw.n), CALL)
 #undef CALL
   if (e != cudaSuccess) return cuda_fail(e, who);
-  const int rc = wait_stream(st, who);
+  const int rc = end_call(scn, st, who);
   if (rc != BF_OK) return rc;
   fill_result(*static_cast<volatile unsigned long long*>(&scn->h_scratch->launch.search.key), scn->desc.n, first, out);
   return BF_OK;
 }
 
 int segment_optimum(const bf_scenario* scn, uint32_t radix, bf_result* out, cudaStream_t st, const char* who) {
+  begin_call(scn);
   const cudaError_t e =
-      bfk::launch_segment_optimum(scn->seg, radix, &scn->d_scratch->launch.seg, scn->d_host_best, st);
+      bfk::launch_segment_optimum(scn->seg, radix, &scn->d_scratch->launch.seg, &scn->d_host_scratch->best, st);
   if (e != cudaSuccess) return cuda_fail(e, who);
-  const int rc = wait_stream(st, who);
+  const int rc = end_call(scn, st, who);
   if (rc != BF_OK) return rc;
   fill_best(*static_cast<volatile bfk::BestRecord*>(&scn->h_scratch->best), scn->desc.n, out);
   return BF_OK;
@@ -478,15 +587,19 @@ int bf_create_scenario(const bf_scenario_desc* desc, bf_scenario** out) {
       s->lt_x = ltrec.x;
     }
   }
-  if (e == cudaSuccess) e = lib_malloc(reinterpret_cast<void**>(&s->d_scratch), kTableOffset + sizeof(uint32_t) * s->seg.entries);
-  if (e == cudaSuccess) e = lib_malloc_host(reinterpret_cast<void**>(&s->h_scratch), sizeof(bf_scratch));
+  ScratchPool::Pair pair{nullptr, nullptr};
+  if (e == cudaSuccess && !g_scratch_pool.take(&pair)) {
+    e = lib_malloc(reinterpret_cast<void**>(&pair.d), sizeof(bf_scratch));
+    if (e == cudaSuccess) e = lib_malloc_host(reinterpret_cast<void**>(&pair.h), sizeof(bf_scratch));
+  }
+  s->d_scratch = pair.d;
+  s->h_scratch = pair.h;
   if (e != cudaSuccess) {
     const int code = cuda_fail(e, "bf_create_scenario");
     if (s->d_scratch) cudaFree(s->d_scratch);
     delete s;
     return code;
   }
-  s->d_table = reinterpret_cast<uint32_t*>(reinterpret_cast<unsigned char*>(s->d_scratch) + kTableOffset);
   s->d_key = &s->d_scratch->key;
   s->h_key = &s->h_scratch->key;
   // The launch states start as (~0, 0, ...) and every launch leaves them so;
@@ -506,8 +619,7 @@ int bf_create_scenario(const bf_scenario_desc* desc, bf_scenario** out) {
     delete s;
     return code;
   }
-  s->d_host_search_key = &static_cast<bf_scratch*>(mirror)->launch.search.key;
-  s->d_host_best = &static_cast<bf_scratch*>(mirror)->best;
+  s->d_host_scratch = static_cast<bf_scratch*>(mirror);
   *out = s;
   return BF_OK;
 }
@@ -516,8 +628,16 @@ int bf_destroy_scenario(bf_scenario* scn) {
   if (!scn) return BF_OK;
   if (scn->d_survivors) cudaFree(scn->d_survivors);
   if (scn->d_levels) cudaFree(scn->d_levels);
-  cudaError_t e1 = scn->d_scratch ? cudaFree(scn->d_scratch) : cudaSuccess;
-  cudaError_t e2 = scn->h_scratch ? cudaFreeHost(scn->h_scratch) : cudaSuccess;
+  cudaError_t e1 = scn->d_table ? cudaFree(scn->d_table) : cudaSuccess, e2 = cudaSuccess;
+  // After a call that failed or stopped waiting, work may still use the scratch:
+  // cudaFree waits for it.
+  int device = -1;
+  const bool here = cudaGetDevice(&device) == cudaSuccess && device == scn->device;
+  if (!here || scn->busy || !g_scratch_pool.keep({scn->d_scratch, scn->h_scratch})) {
+    const cudaError_t e = cudaFree(scn->d_scratch);
+    if (e1 == cudaSuccess) e1 = e;
+    e2 = cudaFreeHost(scn->h_scratch);
+  }
   delete scn;
   if (e1 != cudaSuccess) return cuda_fail(e1, "bf_destroy_scenario");
   if (e2 != cudaSuccess) return cuda_fail(e2, "bf_destroy_scenario");
@@ -539,12 +659,14 @@ int bf_eval_mappings(const bf_scenario* scn, uint64_t first, uint64_t count, uin
   cudaError_t e = cudaSuccess;
   // A captured launch may run after the handle is gone, so it takes the general
   // kernel, whose tables travel by value.  Outside a capture the tables the
-  // sums read outlive the work: bf_destroy_scenario's cudaFree waits for it.
-  if (sums_pay(scn, count) && !is_capturing(st)) {
+  // sums read outlive the work: bf_destroy_scenario frees them by cudaFree, which
+  // waits for it.
+  uint32_t* table = nullptr;
+  if (sums_pay(scn, count) && !is_capturing(st) && segment_tables(scn, &table)) {
     bfk::SegSums sums;
     bfk::host::segment_sums(scn->seg, first, count, &sums);
-    e = bfk::launch_segment_tables(scn->seg, scn->d_table, st);
-    if (e == cudaSuccess) e = bfk::launch_segment_eval(sums, scn->d_table, d_makespan, d_feasible, st);
+    e = bfk::launch_segment_tables(scn->seg, table, st);
+    if (e == cudaSuccess) e = bfk::launch_segment_eval(sums, table, d_makespan, d_feasible, st);
     if (e != cudaSuccess) return cuda_fail(e, "bf_eval_mappings");
     return BF_OK;
   }
@@ -581,12 +703,8 @@ int bf_eval_indices(const bf_scenario* scn, const uint64_t* d_indices, uint64_t 
   if (count == 0) return BF_OK;
   if (!d_indices || !d_makespan || !d_feasible) return fail(BF_EINVAL, "bf_eval_indices: NULL buffer");
   if (const int rc = check_device(scn, "bf_eval_indices")) return rc;
-  int sms = 0;
-  cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, scn->device);
-  if (e != cudaSuccess) return cuda_fail(e, "bf_eval_indices");
-  const uint64_t need = (count + bfk::kThreads - 1) / bfk::kThreads, cap = (uint64_t)sms * 16;
-  const int grid = (int)(need < cap ? need : cap);
-  e = launch_list(scn, d_indices, count, d_makespan, d_feasible, grid, static_cast<cudaStream_t>(cuda_stream));
+  const cudaError_t e =
+      launch_list(scn, d_indices, count, d_makespan, d_feasible, static_cast<cudaStream_t>(cuda_stream));
   if (e != cudaSuccess) return cuda_fail(e, "bf_eval_indices");
   return BF_OK;
 }
@@ -626,13 +744,14 @@ int bf_whatif(const bf_scenario* scn, uint64_t base_index, bf_probe* out, uint32
         h->idx[nc++] = base_index - d[i] * p3[i] + BF_MODE_GPU_NOW * p3[i] + (BF_MODE_GPU_QUEUE - BF_MODE_GPU_NOW) * p3[j];
   }
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  bf_scratch* dv = scn->d_scratch;
-  cudaError_t e = cudaMemcpyAsync(dv->idx, h->idx, sizeof(uint64_t) * nc, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = launch_list(scn, dv->idx, nc, dv->ms, dv->fe, 1 + (int)(nc / bfk::kThreads), st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(h->ms, dv->ms, sizeof(uint32_t) * nc, cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(h->fe, dv->fe, nc, cudaMemcpyDeviceToHost, st);
+  // One launch: the kernel reads the candidates from the pinned host mirror and
+  // writes its results there (a copy in and two copies back took longer than
+  // the kernel: call on a 28-tool workflow 114 -> 88 us).
+  bf_scratch* mirror = scn->d_host_scratch;
+  begin_call(scn);
+  const cudaError_t e = launch_list(scn, mirror->idx, nc, mirror->ms, mirror->fe, st);
   if (e != cudaSuccess) return cuda_fail(e, who);
-  const int rc = wait_stream(st, who);
+  const int rc = end_call(scn, st, who);
   if (rc != BF_OK) return rc;
   // Assemble in Algorithm 1's order.
   uint32_t k = 0, c = 0, sw = n_single;
@@ -713,8 +832,8 @@ int bf_search_pruned(const bf_scenario* scn_const, uint64_t hint_index, bf_resul
     e = lib_malloc(reinterpret_cast<void**>(&scn->d_survivors), sizeof(uint32_t) * scn->pplan.pow3P);
     if (e != cudaSuccess) return cuda_fail(e, who);
   }
-  e = cudaMemcpyAsync(dv->idx, h->idx, sizeof(uint64_t) * nc, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = launch_list(scn, dv->idx, nc, dv->ms, dv->fe, 1, st);
+  begin_call(scn);
+  e = launch_list(scn, scn->d_host_scratch->idx, nc, dv->ms, dv->fe, st);
 
   // 2. Keep the prefixes whose checkpoint bound does not exceed the incumbent;
   //    the filter kernel takes the incumbent from the list kernel's output and
@@ -763,7 +882,7 @@ int bf_search_pruned(const bf_scenario* scn_const, uint64_t hint_index, bf_resul
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(scn->h_key, scn->d_key, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st);
   if (e != cudaSuccess) return cuda_fail(e, who);
-  rc = wait_stream(st, who);
+  rc = end_call(scn, st, who);
   if (rc != BF_OK) return rc;
   fill_result(*scn->h_key, n, 0, out);
   return BF_OK;
@@ -955,43 +1074,6 @@ struct NoAllocDevice {
   cudaStream_t pending_stream = nullptr;
 };
 NoAllocDevice g_noalloc[kNoAllocMaxDevices];
-
-// The driver's cuCtxGetCurrent and cuCtxGetId, looked up through the runtime
-// (the library links no driver library).
-using CtxGetCurrentFn = CUresult (*)(CUcontext*);
-using CtxGetIdFn = CUresult (*)(CUcontext, unsigned long long*);
-struct CtxFns {
-  CtxGetCurrentFn get_current = nullptr;
-  CtxGetIdFn get_id = nullptr;
-};
-
-const CtxFns& ctx_fns() {
-  static const CtxFns fns = [] {
-    CtxFns f;
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      f.get_current = reinterpret_cast<CtxGetCurrentFn>(p);
-    p = nullptr;
-    if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      f.get_id = reinterpret_cast<CtxGetIdFn>(p);
-    return f;
-  }();
-  return fns;
-}
-
-// ID of the current context, 0 when none is current yet.
-int current_ctx_id(unsigned long long* id, const char* who) {
-  const CtxFns& f = ctx_fns();
-  if (!f.get_current || !f.get_id) return fail(BF_ECUDA, "%s: cuCtxGetCurrent/cuCtxGetId not available", who);
-  CUcontext ctx = nullptr;
-  if (f.get_current(&ctx) != CUDA_SUCCESS) return fail(BF_ECUDA, "%s: cuCtxGetCurrent failed", who);
-  *id = 0;
-  if (ctx && f.get_id(ctx, id) != CUDA_SUCCESS) return fail(BF_ECUDA, "%s: cuCtxGetId failed", who);
-  return BF_OK;
-}
 
 // Set-up of the current device, done by the first call on it (and again in a
 // new context after a device reset): the device address of bf_noalloc_scratch.

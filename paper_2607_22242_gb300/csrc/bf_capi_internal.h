@@ -57,7 +57,7 @@ struct bf_scenario {
   bool lanetree;
   uint32_t lt_x, lt_blocks;
   // Scenarios cut by barriers: the segments (seg.count = 0 otherwise), and
-  // their tables behind the device scratch, in the same allocation.
+  // their tables, allocated by the first evaluation that uses them.
   bfk::SegPlan seg;
   uint32_t* d_table;
   int device;
@@ -65,11 +65,11 @@ struct bf_scenario {
   bf_scratch* h_scratch;      // pinned host mirror
   unsigned long long* d_key;  // &d_scratch->key
   unsigned long long* h_key;  // &h_scratch->key
-  unsigned long long* d_host_search_key;  // &h_scratch->launch.search.key as the device addresses it
-  bfk::BestRecord* d_host_best;           // &h_scratch->best as the device addresses it
+  bf_scratch* d_host_scratch; // h_scratch as the device addresses it
   uint32_t* d_survivors;      // pruned search: 3^pplan.P prefix slots, allocated on first use
   uint32_t* d_levels;         // tree search: node buffers of every level, allocated on first use
   size_t levels_bytes;
+  bool busy;                  // a call's work may be in flight (also after one that failed or timed out)
 };
 
 namespace bfcapi {
@@ -83,6 +83,10 @@ cudaError_t lib_malloc(void** p, size_t bytes);
 cudaError_t lib_malloc_host(void** p, size_t bytes);
 // Wait for `st` with the process-wide time limit (BF_ETIMEOUT when it passes).
 int wait_stream(cudaStream_t st, const char* who);
+// Around a handle's call that uses its scratch: work goes out; its last wait,
+// after which (on BF_OK) nothing is in flight.
+void begin_call(const bf_scenario* scn);
+int end_call(const bf_scenario* scn, cudaStream_t st, const char* who);
 // That limit in milliseconds (0: none).
 uint32_t wait_limit_ms();
 // BF_EINVAL unless the handle's device is current.
@@ -92,8 +96,8 @@ int check_device(const bf_scenario* scn, const char* who);
 int segment_optimum(const bf_scenario* scn, uint32_t radix, bf_result* out, cudaStream_t st, const char* who);
 // A best record as a search's result.
 void fill_best(const volatile bfk::BestRecord& best, uint32_t n, bf_result* out);
-// Makespans of a list of mappings on the index-list kernel for the scenario's width.
+// Makespans of a list of mappings on the index-list kernel.
 cudaError_t launch_list(const bf_scenario* scn, const uint64_t* idx, uint64_t count, uint32_t* ms, uint8_t* fe,
-                        int grid, cudaStream_t st);
+                        cudaStream_t st);
 
 }  // namespace bfcapi

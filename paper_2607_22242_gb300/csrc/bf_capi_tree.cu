@@ -86,6 +86,7 @@ int search_tree_impl(const bf_scenario* scn_const, uint32_t space, uint32_t flag
   bf_scratch* h = scn->h_scratch;
   bf_scratch* dv = scn->d_scratch;
   uint32_t launches = 0;
+  begin_call(scn);
 
   // 1. Incumbent: the best feasible of a few mappings of the space (the hint
   //    if it lies in it, all-cpu, all-gpu_now, each tool on its isolated-faster
@@ -108,10 +109,8 @@ int search_tree_impl(const bf_scenario* scn_const, uint32_t space, uint32_t flag
     h->idx[nc++] = now;
     h->idx[nc++] = fast;
     if (R == 3) h->idx[nc++] = 2 * now;
-    e = cudaMemcpyAsync(dv->idx, h->idx, sizeof(uint64_t) * nc, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = launch_list(scn, dv->idx, nc, dv->ms, dv->fe, 1, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h->ms, dv->ms, sizeof(uint32_t) * nc, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h->fe, dv->fe, nc, cudaMemcpyDeviceToHost, st);
+    bf_scratch* mirror = scn->d_host_scratch;
+    e = launch_list(scn, mirror->idx, nc, mirror->ms, mirror->fe, st);
     if (e != cudaSuccess) return cuda_fail(e, who);
     const int rc = wait_stream(st, who);
     if (rc != BF_OK) return rc;
@@ -199,7 +198,7 @@ int search_tree_impl(const bf_scenario* scn_const, uint32_t space, uint32_t flag
   e = cudaMemcpyAsync(&h->best, &dv->best,
                       offsetof(bf_scratch, idx) - offsetof(bf_scratch, best), cudaMemcpyDeviceToHost, st);
   if (e != cudaSuccess) return cuda_fail(e, who);
-  const int rc = wait_stream(st, who);
+  const int rc = end_call(scn, st, who);
   if (rc != BF_OK) return rc;
   if (h->ctr.error) return fail(BF_ECUDA, "%s: internal error 0x%x in the tree kernels", who, h->ctr.error);
   fill_best(h->best, n, out);

@@ -159,36 +159,6 @@ __global__ void __launch_bounds__(kSearchThreads, kSearchMinBlocks) search_kerne
   }
 }
 
-// Index-list evaluation: one mapping per thread (grid-stride), simulated from
-// the start over NP >= n slots.  Indices >= total are flagged 0xFF.
-template <int NP>
-__global__ void __launch_bounds__(kThreads) list_kernel(const __grid_constant__ Tables tb, uint64_t total,
-                                                        const uint64_t* __restrict__ idx, uint64_t count,
-                                                        uint32_t* __restrict__ ms_out, uint8_t* __restrict__ fe_out) {
-  __shared__ SmemTables sd;
-  __shared__ uint32_t rt[ReadyTable<NP>::size];
-  load_smem_tables(tb, sd);
-  fill_ready_table<NP>(tb, rt);
-  __syncthreads();
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; j < count; j += stride) {
-    const uint64_t x = idx[j];
-    uint32_t ms = kInfeasible;
-    uint8_t fe = 0xFFu;
-    if (x < total) {
-      const Digits d = decode((uint32_t)x, tb.n);
-      if ((d.que & tb.big_mask) == 0u) {
-        State<NP> s;
-        init_state(s, tb.all_mask);
-        if (run<NP>(s, tb, sd, rt, d, 0u) == kRunFinished) ms = s.T;
-      }
-      fe = ms != kInfeasible;
-    }
-    ms_out[j] = ms;
-    fe_out[j] = fe;
-  }
-}
-
 // Pruned search, pass 1: one thread per prefix; keeps the prefixes whose
 // checkpoint time plus the tail bound does not exceed the incumbent, the
 // lowest feasible makespan among the ncand candidates the list kernel scored
@@ -312,13 +282,6 @@ cudaError_t BF_PASTE(launch_pruned_search_nw, BF_NW)(const Tables& tb, const Tab
                                                      unsigned long long* key, cudaStream_t st) {
   BF_LAUNCH(pruned_search_kernel, tb.n <= (uint32_t)BF_NW, plan.I, mid_part_words(plan.pow3M), blocks_for(plan), tb,
             tw, plan, survivors, nsurv, key);
-}
-
-// Index lists run the whole scenario in one simulation: this unit handles n <= BF_NW.
-cudaError_t BF_PASTE(launch_list_nw, BF_NW)(const Tables& tb, uint64_t total, const uint64_t* idx, uint64_t count,
-                                            uint32_t* ms, uint8_t* fe, int grid, cudaStream_t st) {
-  list_kernel<BF_NW><<<grid, kThreads, 0, st>>>(tb, total, idx, count, ms, fe);
-  return cudaGetLastError();
 }
 
 }  // namespace bfk

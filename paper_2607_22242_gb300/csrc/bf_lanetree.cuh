@@ -70,33 +70,38 @@ constexpr uint32_t kLtParts = kLtRootParts + 2;  // the root's parts, level [x,y
 constexpr uint32_t kLtStateWords = 9;   // pend and run (16 bits each), qset, qlist (2 words), T, V, tc, gm, tx
 constexpr uint32_t kLtWideStateWords = 12;  // pend and run apart, and the wide queue's second word (2 words)
 
-// State words of a checkpoint in the narrow (W = false) or wide form.
-template <bool W>
+// Form W of the queue: 0 (narrow) up to 16 tools, 1 (wide) up to 24, 2 up to 32 -- one, two or three 64-bit
+// words.  State words of a checkpoint in forms 0 and 1 (2 is for lists of mappings, which have none).
+template <uint32_t W>
 __host__ __device__ constexpr uint32_t lt_state_words() { return W ? kLtWideStateWords : kLtStateWords; }
 
 // 6-bit chunks the tables of an n-tool scenario need.
 __host__ __device__ constexpr uint32_t lt_chunks(uint32_t n) { return (n + kLtChunkBits - 1u) / kLtChunkBits; }
 
-// One scenario of the batch, host-built (bf_plan.h lanetree_record); tools in
-// the renumbered order.
-struct LaneTreeRecord {
+// One scenario of up to CAP tools, host-built (bf_plan.h lanetree_record,
+// lanetree_list_record); tools in the renumbered order.
+template <uint32_t CAP>
+struct LaneTreeRecordT {
   uint32_t n, budget, all_mask, big_mask;  // big_mask: tools with m > M
   uint32_t x, y;                           // level boundaries, 1 <= x <= y <= n
   uint32_t nblocks;                        // batch: blocks the roots [0, 3^x) are split over
   uint32_t pad;
-  uint32_t pred[kLtMaxTools];
-  uint32_t dur[3][kLtMaxTools];  // per mode: c (us); (g + x) * 1024; (l + g + x) * 1024
-  uint32_t vram[kLtMaxTools];
-  uint32_t pv[kLtMaxTools];      // canonical place value 3^orig of each tool
-  uint32_t f[kLtMaxTools + 1];
-  uint64_t frecip[kLtMaxTools + 1];  // floor(2^52 / f[k]) (cpu_advance)
+  uint32_t pred[CAP];
+  uint32_t dur[3][CAP];  // per mode: c (us); (g + x) * 1024; (l + g + x) * 1024
+  uint32_t vram[CAP];
+  uint32_t pv[CAP];      // canonical place value 3^orig of each tool
+  uint32_t f[CAP + 1];
+  uint64_t frecip[CAP + 1];  // floor(2^52 / f[k]) (cpu_advance)
 };
+using LaneTreeRecord = LaneTreeRecordT<kLtMaxTools>;
+using ListRecord = LaneTreeRecordT<32>;  // lists of mappings of up to 32 tools
 
 // Per block: the record and the tables derived from it; NC 6-bit chunks
 // cover the record's tools (NC = lt_chunks(n) or more).
 template <uint32_t NC>
 struct LtSharedT {
-  LaneTreeRecord rec;
+  using Record = LaneTreeRecordT<(NC > 4 ? 32u : kLtMaxTools)>;
+  Record rec;
   uint32_t rt[NC][kLtChunk];  // rt[c][v]: tools whose predecessors in chunk c are all in v
   uint32_t lv[NC][kLtChunk];  // lv[c][v]: VRAM of the tools of chunk c in v
   uint32_t qw[NC][kLtChunk];  // qw[c][v]: isolated gpu_queue times (us) of the tools of chunk c in v, summed
@@ -116,7 +121,8 @@ using LtShared = LtSharedT<2>;  // the batch: up to kLtBatchTools tools
 struct LtState {
   uint32_t pend, run, qset;
   uint64_t qlist;  // waiting queued tools by index, head in bits 0-3 (0-4 wide); qset says how many
-  uint64_t qhi;    // wide form: entries 12 and up, 5 bits each
+  uint64_t qhi;    // wide forms: entries 12 to 23, 5 bits each
+  uint64_t qtop;   // form 2: entries 24 and up
   uint32_t T, V;   // real time (us); virtual GPU clock (1/1024 us of isolated work, modulo 2^32)
   uint32_t tc;     // earliest end of a running CPU tool (0xFFFFFFFF if none)
   uint32_t gm;     // end stamp of the running GPU tool that ends first (when one runs)
@@ -130,7 +136,7 @@ struct LtState {
 // that; a job resumed from a checkpoint starts only tools that were pending
 // there, so it never overwrites the word of a tool running at any checkpoint
 // it or a later job may resume from.  A checkpoint is its state words alone.
-template <bool W = false>
+template <uint32_t W = 0>
 __host__ __device__ inline uint32_t lt_rows(uint32_t n) { return n + 2u * lt_state_words<W>(); }
 
 template <uint32_t NC>
@@ -154,7 +160,7 @@ __device__ __forceinline__ uint32_t lt_sum(const uint32_t (&table)[NC][kLtChunk]
 // Fill the block's tables from S.rec (block-cooperative; S.rec is in place).
 template <uint32_t NC>
 __device__ __forceinline__ void lt_fill_tables(LtSharedT<NC>& S) {
-  const LaneTreeRecord& R = S.rec;
+  const typename LtSharedT<NC>::Record& R = S.rec;
   for (uint32_t e = threadIdx.x; e < NC * kLtChunk; e += blockDim.x) {
     const uint32_t c = e / kLtChunk, v = e % kLtChunk, lo = kLtChunkBits * c;
     uint32_t ready = 0u, mem = 0u, qus = 0u;
@@ -245,10 +251,10 @@ __device__ __forceinline__ void lt_root_modes(const LtSharedT<NC>& S, uint32_t r
 // batch workload from 3.05 to 2.20.  Measured: 16-tool full search 1.59 -> 0.97 ms,
 // an 18-tool layered one 10.8 -> 6.2 ms, batch call of 4096 x 3^10 12.7 ->
 // 11.6 ms.
-template <uint32_t NC, bool W = false>
+template <uint32_t NC, uint32_t W = 0>
 __device__ __forceinline__ uint32_t lt_step(const LtSharedT<NC>& S, LtState& s, uint32_t now, uint32_t que,
                                             uint32_t stop, uint32_t* e, uint32_t stride) {
-  const LaneTreeRecord& R = S.rec;
+  const typename LtSharedT<NC>::Record& R = S.rec;
   const uint32_t gpu = now | que;
   const uint32_t ready = lt_ready(S, s.pend, ~(s.pend | s.run | s.qset));
   if (ready & stop) return kLtStopped;
@@ -272,10 +278,11 @@ __device__ __forceinline__ uint32_t lt_step(const LtSharedT<NC>& S, LtState& s, 
     for (uint32_t m = ready & que; m; m &= m - 1u) {
       const uint32_t i = __ffs(m) - 1u;
       const uint32_t pos = __popc(s.qset);
-      if (W) {  // 12 entries of 5 bits in the first word, the rest in the second
+      if (W) {  // 12 entries of 5 bits in each word
         const uint32_t sh = 5u * pos;
         s.qlist |= pos < 12u ? (uint64_t)i << (sh & 63u) : 0ull;
-        s.qhi |= pos >= 12u ? (uint64_t)i << ((sh - 60u) & 63u) : 0ull;
+        s.qhi |= pos >= 12u && (W < 2u || pos < 24u) ? (uint64_t)i << ((sh - 60u) & 63u) : 0ull;
+        if (W == 2u) s.qtop |= pos >= 24u ? (uint64_t)i << ((sh - 120u) & 63u) : 0ull;
       } else {
         s.qlist |= (uint64_t)i << (4u * pos);
       }
@@ -297,6 +304,10 @@ __device__ __forceinline__ uint32_t lt_step(const LtSharedT<NC>& S, LtState& s, 
       if (W) {
         s.qlist = (s.qlist >> 5) | ((s.qhi & 31ull) << 55);
         s.qhi >>= 5;
+        if (W == 2u) {
+          s.qhi |= (s.qtop & 31ull) << 55;
+          s.qtop >>= 5;
+        }
       } else {
         s.qlist >>= 4;
       }
@@ -366,11 +377,11 @@ __device__ __forceinline__ uint32_t lt_step(const LtSharedT<NC>& S, LtState& s, 
 // the end and reported; a root or a combination none of whose mappings can lie
 // in the range (between its own index part and that plus twice the open tools'
 // place values) is passed over.
-template <uint32_t NC, bool W = false, bool DEAD = false, bool RANGE = false, typename TakeRoot, typename Sink>
+template <uint32_t NC, uint32_t W = 0, bool DEAD = false, bool RANGE = false, typename TakeRoot, typename Sink>
 __device__ __forceinline__ void lt_lane(const LtSharedT<NC>& S, uint32_t* rows, uint32_t stride, TakeRoot take_root,
                                         Sink& sink, uint32_t first = 0u, uint32_t last = 0xFFFFFFFFu) {
   constexpr uint32_t SW = lt_state_words<W>();
-  const LaneTreeRecord& R = S.rec;
+  const typename LtSharedT<NC>::Record& R = S.rec;
   const uint32_t n = R.n;
   uint32_t* const cur = rows;
   const uint32_t stop0 = R.all_mask & ~((1u << R.x) - 1u);
@@ -501,6 +512,34 @@ __device__ __forceinline__ void lt_lane(const LtSharedT<NC>& S, uint32_t* rows, 
       r = kLtFinished;
     }
   }
+}
+
+// The makespan of one mapping simulated whole, kInfeasible if it is.  The
+// record is in the scenario's own numbering with x = min(n, 16), so that its
+// root tables hold the modes of 16 tools in base-81 digits of an index.
+template <uint32_t NC, uint32_t W>
+__device__ __forceinline__ uint32_t lt_whole_mapping(const LtSharedT<NC>& S, uint64_t idx, uint32_t* rows,
+                                                     uint32_t stride) {
+  constexpr uint32_t kRoots = 43046721u;  // 3^16
+  uint32_t now, que, unused;
+  if (S.rec.n <= 16u) {
+    lt_root_modes(S, (uint32_t)idx, &now, &que, &unused);
+  } else {  // the modes of tools 16 and up are those of 0 and up, shifted
+    const uint32_t high = (uint32_t)(idx / kRoots);
+    uint32_t hnow, hque;
+    lt_root_modes(S, high, &hnow, &hque, &unused);
+    lt_root_modes(S, (uint32_t)(idx - (uint64_t)high * kRoots), &now, &que, &unused);
+    now |= hnow << 16;
+    que |= hque << 16;
+  }
+  LtState s{};
+  s.pend = S.rec.all_mask;
+  s.tc = 0xFFFFFFFFu;
+  for (uint32_t steps = 0; steps < S.rec.n + 2u; ++steps) {  // each event retires a tool
+    const uint32_t r = lt_step<NC, W>(S, s, now, que, 0u, rows, stride);
+    if (r != kLtContinue) return r == kLtFinished ? s.T : kInfeasible;
+  }
+  return kStalled;  // never reached by a correct simulation
 }
 
 }  // namespace bfk

@@ -31,6 +31,11 @@ constexpr uint32_t kLtSingleMinTools = 10;
 constexpr uint64_t kLtSingleRootsNum = 1, kLtSingleRootsDen = 2;
 constexpr uint64_t kLtStaticShareNum = 1, kLtStaticShareDen = 2;
 
+// Makespans and flags of a list of `count` >= 1 mappings of up to 32 tools, of
+// the `total` mappings of the space (bf_eval_indices).
+cudaError_t launch_lanetree_list(const TablesT<32>& t, uint64_t total, const uint64_t* idx, uint64_t count,
+                                 uint32_t* ms, uint8_t* fe, cudaStream_t st);
+
 // Blocks of one launch for an n-tool record on the current device: every
 // resident slot of every SM.
 cudaError_t lanetree_single_blocks(uint32_t n, uint32_t* blocks);

@@ -44,8 +44,6 @@ struct SearchSync {
                                  uint8_t* fe, cudaStream_t st);                                     \
   cudaError_t launch_search_nw##NW(const Tables& tb, const Tables& tw, const Plan& plan,             \
                                    SearchSync* sync, unsigned long long* host_key, cudaStream_t st);  \
-  cudaError_t launch_list_nw##NW(const Tables& tb, uint64_t total, const uint64_t* idx, uint64_t count, \
-                                 uint32_t* ms, uint8_t* fe, int grid, cudaStream_t st);             \
   cudaError_t launch_prefix_filter_nw##NW(const Tables& tb, const Plan& plan, const uint32_t* cand_ms,   \
                                           const uint8_t* cand_fe, uint32_t ncand, uint32_t* survivors,   \
                                           uint32_t* count, uint32_t* bound_out, cudaStream_t st);        \

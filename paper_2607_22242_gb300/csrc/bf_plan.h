@@ -742,6 +742,30 @@ inline void lanetree_record(const bf_scenario_desc* d, bfk::LaneTreeRecord* r, u
   }
 }
 
+// Record of an index list: the tools in the scenario's own order, x set so
+// that the root tables cut an index into base-81 digits (lt_whole_mapping).
+template <uint32_t CAP>
+inline void lanetree_list_record(const bfk::TablesT<32>& t, bfk::LaneTreeRecordT<CAP>* r) {
+  std::memset(r, 0, sizeof *r);
+  r->n = t.n;
+  r->budget = t.budget;
+  r->all_mask = t.all_mask;
+  r->big_mask = t.big_mask;
+  r->x = r->y = t.n < kLtRootParts * kLtPartTools ? t.n : kLtRootParts * kLtPartTools;
+  r->nblocks = 1;
+  for (uint32_t v = 0; v < t.n; ++v) {
+    r->pred[v] = t.pred[v];
+    r->dur[0][v] = t.cpu[v];
+    r->dur[1][v] = t.wnow[v];
+    r->dur[2][v] = t.wq[v];
+    r->vram[v] = t.vram[v];
+  }
+  for (uint32_t k = 0; k <= CAP; ++k) {
+    r->f[k] = t.f[k];
+    r->frecip[k] = t.frecip[k];
+  }
+}
+
 // Whether a full search of a scenario goes to the one-scenario lane-tree
 // kernel (sampled cost lt_cost, lanetree_sampled_levels) rather than the
 // search kernel (whole-space tables rt, plan rp, window rw).  The search

@@ -1,5 +1,5 @@
-// bf_tree.cu -- kernels of the tree search (bf_tree.cuh) and the index-list
-// evaluation for scenarios of up to 32 tools.  All state is 32 slots wide.
+// bf_tree.cu -- kernels of the tree search (bf_tree.cuh).  All state is 32 slots
+// wide.
 //
 //   tree_root_kernel   : writes the root node (nothing assigned, T = 0).
 //   tree_expand_kernel : one thread per (parent, mode of the next tool); the
@@ -13,7 +13,6 @@
 //                        checkpoint; compiled for 8..32 slots); per-block best
 //                        (makespan, index) merged into one 16-byte record by
 //                        compare-and-swap.
-//   wide_list_kernel   : makespan of each listed mapping, simulated whole.
 #include <cuda_runtime.h>
 
 #include "bf_launch.h"
@@ -177,47 +176,6 @@ __global__ void __launch_bounds__(LeafShape<NW>::threads, LeafShape<NW>::min_blo
   }
 }
 
-// Digit masks of a canonical index of up to 32 digits.
-__device__ __forceinline__ Digits decode64(uint64_t v, uint32_t n) {
-  Digits d{0u, 0u};
-  for (uint32_t i = 0; i < n; ++i) {
-    const uint64_t q = v / 3u;
-    const uint32_t r = (uint32_t)(v - 3u * q);
-    d.now |= (r == 1u) ? (1u << i) : 0u;
-    d.que |= (r == 2u) ? (1u << i) : 0u;
-    v = q;
-  }
-  return d;
-}
-
-__global__ void __launch_bounds__(kTreeThreads) wide_list_kernel(const __grid_constant__ TablesW tb, uint64_t total,
-                                                                  const uint64_t* __restrict__ idx, uint64_t count,
-                                                                  uint32_t* __restrict__ ms_out,
-                                                                  uint8_t* __restrict__ fe_out) {
-  __shared__ SmemTablesW sd;
-  __shared__ uint32_t rt[ReadyTable<kTreeSlots>::size];
-  load_smem_tables(tb, sd);
-  fill_ready_table<kTreeSlots>(tb, rt);
-  __syncthreads();
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; j < count; j += stride) {
-    const uint64_t x = idx[j];
-    uint32_t ms = kInfeasible;
-    uint8_t fe = 0xFFu;
-    if (x < total) {
-      const Digits d = decode64(x, tb.n);
-      if ((d.que & tb.big_mask) == 0u) {
-        State<kTreeSlots> s;
-        init_state(s, tb.all_mask);
-        if (run<kTreeSlots>(s, tb, sd, rt, d, 0u) == kRunFinished) ms = s.T;
-      }
-      fe = ms != kInfeasible;
-    }
-    ms_out[j] = ms;
-    fe_out[j] = fe;
-  }
-}
-
 }  // namespace
 
 size_t tree_node_words() { return (size_t)kNW; }
@@ -276,12 +234,6 @@ cudaError_t launch_tree_leaf(const TablesW& tb, const TreeConsts& tc, const uint
   BF_TREE_BUCKETS(BF_TRY)
 #undef BF_TRY
   return cudaErrorInvalidValue;
-}
-
-cudaError_t launch_wide_list(const TablesW& tb, uint64_t total, const uint64_t* idx, uint64_t count, uint32_t* ms,
-                             uint8_t* fe, int grid, cudaStream_t st) {
-  wide_list_kernel<<<grid, kTreeThreads, 0, st>>>(tb, total, idx, count, ms, fe);
-  return cudaGetLastError();
 }
 
 }  // namespace bfk

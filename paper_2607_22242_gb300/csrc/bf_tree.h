@@ -34,7 +34,5 @@ cudaError_t launch_tree_expand(const TablesW& tb, const TreeConsts& tc, const ui
 cudaError_t launch_tree_leaf(const TablesW& tb, const TreeConsts& tc, const uint32_t* src, uint32_t src_cap,
                              uint32_t lo, uint32_t cnt, uint32_t target_tasks, uint32_t* bound, BestRecord* best,
                              TreeCounters* ctr, cudaStream_t st);
-cudaError_t launch_wide_list(const TablesW& tb, uint64_t total, const uint64_t* idx, uint64_t count, uint32_t* ms,
-                             uint8_t* fe, int grid, cudaStream_t st);
 
 }  // namespace bfk

@@ -1,0 +1,67 @@
+"""Handles made and destroyed one after the other, and by several threads at once, share pooled scratch (GPU)."""
+import threading
+
+import pytest
+
+import oracle
+from paper_2607_22242_gb300 import bf
+from paper_2607_22242_gb300 import scenarios as S
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("threads,rounds", [(1, 40), (6, 25)])
+def test_handles_in_turn(threads, rounds):
+    """More handles than the pool keeps, of every kind of search, each result the oracle's: no launch state or record
+    of an earlier handle is left in the scratch of a later one."""
+    import numpy as np
+    import torch
+    rng = np.random.default_rng(threads)
+    scns = [S.random_small(rng, int(n), edge_p=0.3) for n in rng.integers(2, 11, 12)]
+    scns += [S.random_segmented(rng, 9), S.config0()]
+    want = [oracle.search(s) for s in scns]
+    errors = []
+
+    def work(t):
+        try:
+            stream = torch.cuda.Stream()
+            held = []
+            for k in range(rounds):
+                j = (k * 5 + t) % len(scns)
+                h = bf.create_scenario(scns[j])
+                held.append(h)
+                for r in (bf.search_best(h, stream), bf.search_pruned(h, None, stream),
+                          bf.search_tree(h, bf.SPACE_FULL, True, None, stream)[0]):
+                    if (r.index, r.makespan_us) != want[j]:
+                        errors.append((t, k, j, r))
+                if len(held) > 4:
+                    held.pop(0).close()
+            for h in held:
+                h.close()
+        except Exception as e:  # noqa: BLE001
+            errors.append((t, e))
+    ts = [threading.Thread(target=work, args=(t,)) for t in range(threads)]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join(timeout=120)
+    assert not any(t.is_alive() for t in ts) and errors == []
+
+
+@pytest.mark.gpu
+def test_a_handle_closed_after_a_timeout_keeps_its_scratch_to_itself():
+    """A one-off search whose wait runs out closes its handle with the kernel still running: the next handles get
+    other scratch, and their results are right."""
+    import torch
+    scn, small = S.config3(), S.config0()
+    bf.set_wait_timeout_ms(1)
+    try:
+        with pytest.raises(bf.BfError) as ei:
+            bf.search_best(scn)
+        assert ei.value.code == bf.BF_ETIMEOUT
+        bf.set_wait_timeout_ms(600000)
+        for _ in range(3):
+            r = bf.search_best(small)
+            assert (r.index, r.makespan_us) == oracle.search(small)
+    finally:
+        bf.set_wait_timeout_ms(600000)
+        torch.cuda.synchronize()
