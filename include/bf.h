@@ -237,8 +237,10 @@ typedef struct bf_tree_stats {
  * its mode (or min(c, g + x) if open), and queued tools run one at a time.
  * The first bound is the best of a few mappings of the space (hint_index if
  * it lies in it, all-cpu, all-gpu_now, each tool on its isolated-faster
- * device, all-gpu_queue); when the tree is large, a narrow dive to the leaves
- * (8192 nodes per level) tightens it before the search restarts from the root;
+ * device, all-gpu_queue); when the tree is large, two narrow dives to the leaves
+ * (256, then 2048 nodes per level) tighten it before the search restarts from the
+ * root; at the leaves, modes in which a tool would end too late for the bound are
+ * not enumerated;
  * better bounds are found as the search proceeds.  space: BF_SPACE_FULL or
  * BF_SPACE_BINARY.
  * flags: 0 or BF_TREE_NO_PRUNE (every mapping of the space is simulated:

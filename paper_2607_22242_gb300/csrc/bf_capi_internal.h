@@ -30,8 +30,8 @@ struct bf_scratch {
   bfk::BestRecord best;      // tree search: best (makespan, index) so far
   uint32_t bound;            // tree search: makespan bound for pruning
   uint32_t pad2;
-  unsigned long long appended;  // tree search: nodes appended by all expansions so far
   bfk::TreeCounters ctr;     // tree search: counters and error bits
+  uint32_t count[BF_MAX_TOOLS + 1];  // tree search: nodes of each level
   uint64_t idx[BF_MAX_PROBES];
   uint32_t ms[BF_MAX_PROBES];
   uint8_t fe[BF_MAX_PROBES];

@@ -18,6 +18,9 @@ using bfk::host::pow3;
 
 namespace {
 
+// The tree search's record, bound, counters and level sizes, copied together.
+constexpr size_t kTreeStateBytes = offsetof(bf_scratch, idx) - offsetof(bf_scratch, best);
+
 int search_tree_impl(const bf_scenario* scn_const, uint32_t space, uint32_t flags, uint64_t hint_index,
                      bf_result* out, bf_tree_stats* stats, void* cuda_stream) {
   const char* who = "bf_search_tree";
@@ -81,18 +84,29 @@ int search_tree_impl(const bf_scenario* scn_const, uint32_t space, uint32_t flag
     if (e != cudaSuccess) return cuda_fail(e, who);
     scn->levels_bytes = need;
   }
-  auto level = [&](uint32_t d) { return scn->d_levels + level_words * d; };
+
+  auto tree_level = [&](uint32_t d) { return bfk::TreeLevel{scn->d_levels + level_words * d, scn->d_scratch->count + d}; };
 
   bf_scratch* h = scn->h_scratch;
   bf_scratch* dv = scn->d_scratch;
   uint32_t launches = 0;
   begin_call(scn);
 
-  // 1. Incumbent: the best feasible of a few mappings of the space (the hint
+  // 1. Reset the record, bound, counters and level sizes (pinned, and not
+  //    written again before the first wait below).
+  h->best.ms = ~0ull;
+  h->best.idx = ~0ull;
+  h->bound = 0xFFFFFFFFu;
+  std::memset(&h->ctr, 0, sizeof h->ctr);
+  h->ctr.incumbent = 0xFFFFFFFFu;
+  std::memset(h->count, 0, sizeof h->count);
+  e = cudaMemcpyAsync(&dv->best, &h->best, kTreeStateBytes, cudaMemcpyHostToDevice, st);
+
+  // 2. Incumbent: the best feasible of a few mappings of the space (the hint
   //    if it lies in it, all-cpu, all-gpu_now, each tool on its isolated-faster
-  //    device, and all-gpu_queue in the full space).
-  uint32_t bound = 0xFFFFFFFFu;
-  if (prune) {
+  //    device, and all-gpu_queue in the full space), scored and compared on the
+  //    device.
+  if (prune && e == cudaSuccess) {
     const uint64_t total = pow3(n);
     uint32_t nc = 0;
     bool hint_ok = hint_index < total;
@@ -109,106 +123,103 @@ int search_tree_impl(const bf_scenario* scn_const, uint32_t space, uint32_t flag
     h->idx[nc++] = now;
     h->idx[nc++] = fast;
     if (R == 3) h->idx[nc++] = 2 * now;
-    bf_scratch* mirror = scn->d_host_scratch;
-    e = launch_list(scn, mirror->idx, nc, mirror->ms, mirror->fe, st);
-    if (e != cudaSuccess) return cuda_fail(e, who);
-    const int rc = wait_stream(st, who);
-    if (rc != BF_OK) return rc;
-    ++launches;
-    for (uint32_t j = 0; j < nc; ++j)
-      if (h->fe[j] == 1 && h->ms[j] < bound) bound = h->ms[j];
+    e = launch_list(scn, scn->d_host_scratch->idx, nc, dv->ms, dv->fe, st);
+    if (e == cudaSuccess) e = bfk::launch_tree_bound(dv->ms, dv->fe, nc, &dv->bound, &dv->ctr, st);
+    launches += 2;
   }
-
-  // 2. Reset the record, bound and counters; write the root node.
-  h->best.ms = ~0ull;
-  h->best.idx = ~0ull;
-  h->bound = bound;
-  h->appended = 0;
-  std::memset(&h->ctr, 0, sizeof h->ctr);
-  e = cudaMemcpyAsync(&dv->best, &h->best,
-                      offsetof(bf_scratch, idx) - offsetof(bf_scratch, best), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = bfk::launch_tree_root(tb, level(0), cap, st);
   if (e != cudaSuccess) return cuda_fail(e, who);
-  ++launches;
 
-  // 3. Depth first over levels: pop up to kPop nodes (a whole leaf-level
-  //    buffer) from the deepest non-empty level, and expand them into the
-  //    next level or enumerate their leaves.  A large tree starts with a
-  //    dive: pops of kDive nodes reach the leaves after one expansion per
-  //    level, and the first leaves' makespans become the bound; the dive's
-  //    other nodes are then dropped and the search restarts from the root
-  //    (the root stays in the level-0 buffer), now pruning the wide levels
-  //    with that bound.  (Measured: 8192 beat 64 and 1024, and beat diving
-  //    without the restart.)
-  constexpr uint32_t kDive = 8192;
+  // 3. Depth first over levels, in chains of launches that the host does not
+  //    wait between: from the deepest level that holds nodes, up to `pop` nodes
+  //    of it are expanded into the next level, up to `pop` of those (all of the
+  //    leaf level) into the one after, and so on to the leaves; after the
+  //    chain the host reads how many nodes each level has kept.  The levels
+  //    below the one a chain starts from are empty.  The first chain starts
+  //    with every combination of the first d0 tools.  A large tree starts with
+  //    two dives, chains of kDives[i] nodes per level, whose leaves set the
+  //    bound; their other nodes are then dropped and the search starts over with
+  //    that bound.  Over 12 layered and sparse DAGs of 8 to 26 tools, dives of
+  //    {256, 2048} nodes took 0.88 times the 8192 of a single dive on average
+  //    ({256, 8192} 0.91, {1024, 8192} 0.92, {1024} 0.95, {64, 8192} 1.06).
+  //    With these chains and the leaf modes (bf_tree.cuh node_leaf_modes) full
+  //    searches went from 2.30 to 1.28 ms (18 layered tools), 4.06 to 1.83 (20),
+  //    7.4 to 2.1 (24) and 6.4 to 2.1 ms (26).
+  static constexpr uint32_t kDives[] = {256, 2048};
+  constexpr uint32_t kStart = 8192;
   // The whole search, not only each wait, is held to the wait limit.
   const auto t_start = std::chrono::steady_clock::now();
   const uint32_t limit_ms = wait_limit_ms();
-  std::vector<uint32_t> size(levels, 0);
-  size[0] = 1;
-  uint64_t nodes = 1;
-  uint64_t leaf_level_nodes = 1;  // radix^L, saturating
+  uint32_t d0 = 0;
+  uint64_t start_nodes = 1, leaf_level_nodes = 1;  // radix^d0; radix^L, saturating
+  while (d0 < tc.leaf_level && start_nodes * R <= kStart) {
+    start_nodes *= R;
+    ++d0;
+  }
   for (uint32_t i = 0; i < tc.leaf_level && leaf_level_nodes <= kPop; ++i) leaf_level_nodes *= R;
-  bool diving = prune && leaf_level_nodes > kPop;
-  for (;;) {
-    int d = (int)levels - 1;
-    while (d >= 0 && size[d] == 0) --d;
-    if (d < 0) break;
-    const uint32_t L = (uint32_t)d;
-    const uint32_t pop = diving ? kDive : kPop;
-    const uint32_t take = L == tc.leaf_level ? size[L] : (size[L] < pop ? size[L] : pop);
-    if (diving && L == tc.leaf_level) {
-      e = bfk::launch_tree_leaf(tb, tc, level(L), cap, size[L] - take, take, 16384, &dv->bound, &dv->best, &dv->ctr,
-                                st);
-      if (e != cudaSuccess) return cuda_fail(e, who);
+  auto chain = [&](uint32_t from, uint64_t most, uint32_t pop) {  // most: nodes level `from` may hold
+    for (uint32_t d = from; d < tc.leaf_level && e == cudaSuccess; ++d) {
+      e = bfk::launch_tree_expand(tb, tc, tree_level(d), pop, (uint32_t)most, d, tree_level(d + 1), cap, &dv->bound,
+                                  &dv->ctr, st);
+      most = (most < pop ? most : pop) * R;
       ++launches;
-      std::fill(size.begin(), size.end(), 0u);
-      size[0] = 1;
-      diving = false;
-      continue;
     }
-    const uint32_t lo = size[L] - take;
-    size[L] = lo;
-    if (L == tc.leaf_level) {
-      e = bfk::launch_tree_leaf(tb, tc, level(L), cap, lo, take, 16384, &dv->bound, &dv->best, &dv->ctr, st);
-      if (e != cudaSuccess) return cuda_fail(e, who);
-      ++launches;
-      continue;
-    }
-    const unsigned long long before = h->appended;
-    e = bfk::launch_tree_expand(tb, tc, level(L), cap, lo, take, L, level(L + 1), cap, &dv->appended, before,
-                                &dv->bound, &dv->ctr, st);
     if (e == cudaSuccess)
-      e = cudaMemcpyAsync(&h->appended, &dv->appended, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st);
+      e = bfk::launch_tree_leaf(tb, tc, tree_level(tc.leaf_level), cap, (uint32_t)most, &dv->bound, &dv->best,
+                                &dv->ctr, st);
+    ++launches;
+  };
+  auto start = [&]() {
+    e = bfk::launch_tree_start(tb, tc, d0, tree_level(d0), cap, &dv->bound, &dv->ctr, st);
+    ++launches;
+  };
+  start();
+  if (prune && leaf_level_nodes > kPop && e == cudaSuccess) {
+    for (const uint32_t pop : kDives) {
+      if (e == cudaSuccess) chain(d0, start_nodes, pop);
+      if (e == cudaSuccess) e = cudaMemsetAsync(dv->count, 0, sizeof dv->count, st);
+      if (e == cudaSuccess) start();
+    }
+  }
+  std::vector<uint32_t> size(levels, 0);
+  uint32_t from = d0;
+  uint64_t most = start_nodes;
+  for (;;) {
+    if (e == cudaSuccess) chain(from, most, kPop);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(h->count, dv->count, sizeof h->count, cudaMemcpyDeviceToHost, st);
     if (e != cudaSuccess) return cuda_fail(e, who);
     const int rc = wait_stream(st, who);
     if (rc != BF_OK) return rc;
+    // What each level of the chain has kept: all but the last kPop nodes.
+    for (uint32_t d = from; d < tc.leaf_level; ++d) size[d] = h->count[d] > kPop ? h->count[d] - kPop : 0u;
+    int d = (int)tc.leaf_level - 1;
+    while (d >= 0 && size[d] == 0) --d;
+    if (d < 0) break;
     if (limit_ms) {
       const auto ms = std::chrono::duration_cast<std::chrono::milliseconds>(std::chrono::steady_clock::now() - t_start);
       if (ms.count() > (long long)limit_ms)
         return fail(BF_ETIMEOUT, "%s: search not finished after %u ms", who, limit_ms);
     }
-    ++launches;
-    const uint32_t added = (uint32_t)(h->appended - before);
-    size[L + 1] = added;
-    nodes += added;
+    from = (uint32_t)d;
+    most = size[d];
+    for (uint32_t i = 0; i < levels; ++i) h->count[i] = i <= from ? size[i] : 0u;
+    e = cudaMemcpyAsync(dv->count, h->count, sizeof h->count, cudaMemcpyHostToDevice, st);
   }
 
   // 4. The record.
-  e = cudaMemcpyAsync(&h->best, &dv->best,
-                      offsetof(bf_scratch, idx) - offsetof(bf_scratch, best), cudaMemcpyDeviceToHost, st);
+  e = cudaMemcpyAsync(&h->best, &dv->best, kTreeStateBytes, cudaMemcpyDeviceToHost, st);
   if (e != cudaSuccess) return cuda_fail(e, who);
   const int rc = end_call(scn, st, who);
   if (rc != BF_OK) return rc;
   if (h->ctr.error) return fail(BF_ECUDA, "%s: internal error 0x%x in the tree kernels", who, h->ctr.error);
   fill_best(h->best, n, out);
   if (stats) {
-    stats->nodes = nodes;
+    stats->nodes = 1 + h->ctr.nodes;
     stats->leaf_nodes = h->ctr.leaf_nodes;
     stats->leaves = h->ctr.leaves;
     stats->launches = launches;
     stats->leaf_depth = tc.D;
-    stats->incumbent_us = bound;
+    stats->incumbent_us = h->ctr.incumbent;
   }
   return BF_OK;
 }

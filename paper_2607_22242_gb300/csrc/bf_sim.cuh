@@ -286,12 +286,15 @@ __device__ __forceinline__ uint32_t ready_of(const uint32_t* table, uint32_t pen
 // `join`, a subset of stop_mask: tools that wait for every other tool.  They do
 // not hold the closed form back; the run then reports kRunStopped at the
 // instant they become ready, with s.T and s.done set and nothing else.
+// `limit`: a run whose time passes it is given up as infeasible (branch and
+// bound: its makespan cannot be the best).
 // Measured: 19-tool search 15.7 -> 11.2 ms, 12-tool fan-out/fan-in 64 -> 55 us;
 // no change where a warp's lanes diverge and its slowest one sets the pace
 // (16-tool layered ranges and lists, 1 to 3 %).
 template <int NT, typename TB, typename SD>
 __device__ __forceinline__ uint32_t run(State<NT>& s, const TB& tb, const SD& sd, const uint32_t* ready_table,
-                                        Digits dg, uint32_t stop_mask, uint32_t join = 0u) {
+                                        Digits dg, uint32_t stop_mask, uint32_t join = 0u,
+                                        uint32_t limit = 0xFFFFFFFFu) {
   static_assert(NT <= TB::cap, "state wider than its tables");
   const uint32_t cpu_mask = tb.all_mask & ~(dg.now | dg.que);
 #pragma unroll 1
@@ -392,6 +395,7 @@ __device__ __forceinline__ uint32_t run(State<NT>& s, const TB& tb, const SD& sd
     } else {
       s.T = s.tc;
     }
+    if (s.T > limit) return kRunInfeasible;
 
     // ---- retire everything that ends at T ------------------------------------
     if (s.tc == s.T) {

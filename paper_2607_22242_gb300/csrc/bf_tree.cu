@@ -1,18 +1,25 @@
 // bf_tree.cu -- kernels of the tree search (bf_tree.cuh).  All state is 32 slots
 // wide.
 //
-//   tree_root_kernel   : writes the root node (nothing assigned, T = 0).
+//   tree_bound_kernel  : the starting bound from the scored candidates.
+//   tree_start_kernel  : one thread per combination of the first d0 tools'
+//                        modes, simulated from time 0, bounded and appended to
+//                        level d0 (one launch instead of d0 small ones).
 //   tree_expand_kernel : one thread per (parent, mode of the next tool); the
 //                        child is resumed to its checkpoint, bounded, and the
 //                        survivors are appended to the next level's buffer
-//                        (one atomicAdd per warp on a running total).
+//                        (one atomicAdd per warp on the level's count).
 //   tree_leaf_kernel   : one warp per 32 leaf-level nodes (one per lane) and a
 //                        chunk of the radix^D combinations of the last D tools,
-//                        walked in lockstep over the leaf window (tools from the
+//                        walked over the leaf window (tools from the
 //                        lowest one that can still be running at a leaf
-//                        checkpoint; compiled for 8..32 slots); per-block best
+//                        checkpoint; compiled for 8..32 slots), without those
+//                        in which a leaf tool must end too late; per-block best
 //                        (makespan, index) merged into one 16-byte record by
 //                        compare-and-swap.
+//
+// Level sizes stay on the device: the launches of a chain of levels are sized
+// for the most nodes a level can hold and read how many there are.
 #include <cuda_runtime.h>
 
 #include "bf_launch.h"
@@ -30,49 +37,85 @@ __device__ __forceinline__ uint32_t read_bound(const uint32_t* bound) {
   return *reinterpret_cast<const volatile uint32_t*>(bound);
 }
 
-__global__ void tree_root_kernel(const __grid_constant__ TablesW tb, uint32_t* buf, uint32_t cap) {
-  State<kTreeSlots> s;
-  init_state(s, tb.all_mask);
-  store_node(s, Digits{0u, 0u}, buf, cap, 0u);
+__device__ __forceinline__ uint32_t read_count(const uint32_t* count) {
+  return *reinterpret_cast<const volatile uint32_t*>(count);
 }
 
-__global__ void __launch_bounds__(kTreeThreads, 2) tree_expand_kernel(
-    const __grid_constant__ TablesW tb, const __grid_constant__ TreeConsts tc, const uint32_t* __restrict__ src,
-    uint32_t src_cap, uint32_t lo, uint32_t cnt, uint32_t d, uint32_t* __restrict__ dst, uint32_t dst_cap,
-    unsigned long long* appended, unsigned long long base_total, const uint32_t* bound, TreeCounters* ctr) {
+__global__ void tree_bound_kernel(const uint32_t* ms, const uint8_t* fe, uint32_t n, uint32_t* bound,
+                                  TreeCounters* ctr) {
+  uint32_t b = kInfeasible;
+  for (uint32_t j = 0; j < n; ++j)
+    if (fe[j] == 1u && ms[j] < b) b = ms[j];
+  *bound = b;
+  ctr->incumbent = b;
+}
+
+// Append this lane's node (if it keeps one) to a level: a slot per lane from
+// one atomicAdd per warp.
+__device__ __forceinline__ void append_node(bool keep, const State<kTreeSlots>& s, Digits dg, TreeLevel dst,
+                                            uint32_t cap, TreeCounters* ctr) {
+  const uint32_t ballot = __ballot_sync(0xFFFFFFFFu, keep);
+  if (ballot == 0u) return;
+  const uint32_t lane = threadIdx.x & 31u, leader = __ffs(ballot) - 1;
+  uint32_t base = 0u;
+  if (lane == leader) {
+    base = atomicAdd(dst.count, (uint32_t)__popc(ballot));
+    atomicAdd(&ctr->nodes, (unsigned long long)__popc(ballot));
+  }
+  base = __shfl_sync(0xFFFFFFFFu, base, leader);
+  if (!keep) return;
+  const uint32_t slot = base + __popc(ballot & ((1u << lane) - 1u));
+  if (slot >= cap) {  // cannot happen (nodes * radix <= cap); recorded, never written
+    atomicOr(&ctr->error, 1u);
+    return;
+  }
+  store_node(s, dg, dst.buf, cap, slot);
+}
+
+__global__ void __launch_bounds__(kTreeThreads, 2) tree_start_kernel(
+    const __grid_constant__ TablesW tb, const __grid_constant__ TreeConsts tc, uint32_t d0, uint32_t combos,
+    TreeLevel dst, uint32_t cap, const uint32_t* bound, TreeCounters* ctr) {
   __shared__ SmemTablesW sd;
   __shared__ uint32_t rt[ReadyTable<kTreeSlots>::size];
   __shared__ uint32_t ef[kTreeSlots * kTreeThreads];  // forward_bound scratch, [tool][thread]
   load_smem_tables(tb, sd);
   fill_ready_table<kTreeSlots>(tb, rt);
   __syncthreads();
+  const uint32_t p = blockIdx.x * kTreeThreads + threadIdx.x;
+  State<kTreeSlots> s;
+  Digits dg{0u, 0u};
+  bool keep = false;
+  if (p < combos) {
+    dg = leaf_digits(p, tc.radix, d0, 0u);
+    init_state(s, tb.all_mask);
+    keep = expand_start<kTreeSlots>(tb, sd, rt, tc, s, dg, d0, read_bound(bound), ef + threadIdx.x, kTreeThreads);
+  }
+  append_node(keep, s, dg, dst, cap, ctr);
+}
+
+__global__ void __launch_bounds__(kTreeThreads, 2) tree_expand_kernel(
+    const __grid_constant__ TablesW tb, const __grid_constant__ TreeConsts tc, TreeLevel src, uint32_t pop, uint32_t d,
+    TreeLevel dst, uint32_t cap, const uint32_t* bound, TreeCounters* ctr) {
+  __shared__ SmemTablesW sd;
+  __shared__ uint32_t rt[ReadyTable<kTreeSlots>::size];
+  __shared__ uint32_t ef[kTreeSlots * kTreeThreads];  // forward_bound scratch, [tool][thread]
   // Thread t: mode a = t / cnt of tool d for parent lo + t % cnt, so that a
   // warp's lanes hold neighbouring parents with the same new mode.
+  const uint32_t size = read_count(src.count), cnt = min(size, pop), lo = size - cnt;
+  if (blockIdx.x * kTreeThreads >= cnt * tc.radix) return;
+  load_smem_tables(tb, sd);
+  fill_ready_table<kTreeSlots>(tb, rt);
+  __syncthreads();
   const uint32_t t = blockIdx.x * kTreeThreads + threadIdx.x;
-  const uint32_t a = t / max(cnt, 1u), j = t - a * cnt;
+  const uint32_t a = t / cnt, j = t - a * cnt;
   bool keep = false;
   State<kTreeSlots> s;
   Digits dg{0u, 0u};
   if (a < tc.radix) {
-    load_node(src, src_cap, lo + j, s, dg);
+    load_node(src.buf, cap, lo + j, s, dg);
     keep = expand_child<kTreeSlots>(tb, sd, rt, tc, s, dg, d, a, read_bound(bound), ef + threadIdx.x, kTreeThreads);
   }
-  const uint32_t ballot = __ballot_sync(0xFFFFFFFFu, keep);
-  if (ballot == 0u) return;
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t leader = __ffs(ballot) - 1;
-  // `appended` counts every node appended by every expansion of this search;
-  // this launch's children get slots from base_total (its value at launch) on.
-  unsigned long long base = 0ull;
-  if (lane == leader) base = atomicAdd(appended, (unsigned long long)__popc(ballot));
-  base = __shfl_sync(0xFFFFFFFFu, base, leader);
-  if (!keep) return;
-  const uint64_t slot = (base - base_total) + (uint64_t)__popc(ballot & ((1u << lane) - 1u));
-  if (slot >= dst_cap) {  // cannot happen (cnt * radix <= dst_cap); recorded, never written
-    atomicOr(&ctr->error, 1u);
-    return;
-  }
-  store_node(s, dg, dst, dst_cap, (uint32_t)slot);
+  append_node(keep, s, dg, dst, cap, ctr);
 }
 
 // Lexicographic (makespan, index) minimum of the 16-byte record at *p.  Every
@@ -110,49 +153,56 @@ struct LeafShape {
   static constexpr int min_blocks = NW <= 12 ? 4 : NW <= 16 ? 6 : NW <= 24 ? 5 : 4;
 };
 
+// Warp tasks are 32 nodes times a chunk of combinations: about
+// kTreeLeafTasks of them over all nodes, at least 16 combinations each, taken
+// in turn by the grid's warps.
+constexpr uint32_t kTreeLeafTasks = 16384;
+
 template <int NW>
 __global__ void __launch_bounds__(LeafShape<NW>::threads, LeafShape<NW>::min_blocks) tree_leaf_kernel(
     const __grid_constant__ TablesW tb, const __grid_constant__ TablesT<NW> tw, const __grid_constant__ TreeConsts tc,
-    const uint32_t* __restrict__ src, uint32_t src_cap, uint32_t lo, uint32_t cnt, uint32_t parts, uint32_t chunk,
-    uint32_t* bound, BestRecord* best, TreeCounters* ctr) {
+    TreeLevel src, uint32_t cap, uint32_t* bound, BestRecord* best, TreeCounters* ctr) {
   extern __shared__ uint32_t lane_state[];
   __shared__ SmemTablesT<NW> sdw;
   __shared__ uint32_t rtw[ReadyTable<NW>::size];
   __shared__ uint32_t wb_ms[LeafShape<NW>::warps], wb_now[LeafShape<NW>::warps], wb_que[LeafShape<NW>::warps];
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  const uint32_t cnt = read_count(src.count), groups = (cnt + 31u) / 32u;
+  // With a lone last tool, combinations cover the leaf tools but the last
+  // one, each standing for radix mappings.
+  const uint32_t ncomb = tc.alone_last ? tc.combos / tc.radix : tc.combos;
+  const uint32_t want = min((kTreeLeafTasks + groups - 1u) / max(groups, 1u), (ncomb + 15u) / 16u);
+  const uint32_t chunk = (ncomb + max(want, 1u) - 1u) / max(want, 1u), parts = (ncomb + chunk - 1u) / chunk;
+  if (blockIdx.x * LeafShape<NW>::warps >= groups * parts) return;
   load_smem_tables(tw, sdw);
   fill_ready_table<NW>(tw, rtw);
   __syncthreads();
-  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-  const uint32_t task = blockIdx.x * LeafShape<NW>::warps + warp;
-  const uint32_t groups = (cnt + 31u) / 32u;
   LaneBest lb;
-  if (task < groups * parts) {
-    const uint32_t g = task / parts, part = task - g * parts;
-    const uint32_t j = g * 32u + lane;
+  uint32_t* const slot = lane_state + threadIdx.x;
+  for (uint32_t task = blockIdx.x * LeafShape<NW>::warps + warp; task < groups * parts;
+       task += gridDim.x * LeafShape<NW>::warps) {
+    const uint32_t g = task / parts, part = task - g * parts, j = g * 32u + lane;
     bool valid = j < cnt;
     Digits dg{0u, 0u};
-    uint32_t* slot = lane_state + threadIdx.x;
+    LeafModes modes{~0u, ~0u, ~0u};
+    const uint32_t limit = tc.prune ? read_bound(bound) : kInfeasible;
     if (valid) {
-      const uint32_t* t = src + lo + j + (size_t)(2 * kTreeSlots) * src_cap;
-      dg = Digits{t[9 * (size_t)src_cap], t[10 * (size_t)src_cap]};
-      // the incumbent may have improved since this node was bounded
-      if (tc.prune &&
-          node_lower_bound(src, src_cap, lo + j, tb, tc, dg, tb.all_mask >> tc.D) > (uint64_t)read_bound(bound))
-        valid = false;
-      else
-        node_to_window<NW>(src, src_cap, lo + j, tc.W0, tw.n, slot, LeafShape<NW>::threads);
+      const uint32_t* t = src.buf + j + (size_t)(2 * kTreeSlots) * cap;
+      dg = Digits{t[9 * (size_t)cap], t[10 * (size_t)cap]};
+      // The incumbent may have improved since this node was bounded; only modes
+      // within it are enumerated.
+      if (tc.prune) valid = node_leaf_modes(src.buf, cap, j, tb, tc, dg, limit, slot, LeafShape<NW>::threads, &modes);
+      if (valid) node_to_window<NW>(src.buf, cap, j, tc.W0, tw.n, slot, LeafShape<NW>::threads);
     }
-    const uint32_t ran = __ballot_sync(0xFFFFFFFFu, valid);
-    // With a lone last tool, combinations cover the leaf tools but the last
-    // one, each standing for radix mappings.
-    const uint32_t ncomb = tc.alone_last ? tc.combos / tc.radix : tc.combos;
-    const uint32_t c0 = part * chunk;
-    const uint32_t c1 = min(c0 + chunk, ncomb);
-    if (lane == 0 && ran) {
-      if (part == 0) atomicAdd(&ctr->leaf_nodes, (unsigned long long)__popc(ran));
-      atomicAdd(&ctr->leaves, (unsigned long long)__popc(ran) * (c1 - c0) * (tc.alone_last ? tc.radix : 1u));
+    const uint32_t nodes = __ballot_sync(0xFFFFFFFFu, valid);
+    if (nodes == 0u) continue;
+    const uint32_t c0 = part * chunk, c1 = min(c0 + chunk, ncomb);
+    const uint32_t ran = leaf_combos<NW>(tw, sdw, rtw, tc, slot, LeafShape<NW>::threads, dg, valid, c0, c1, lb, modes, limit);
+    const uint32_t all = __reduce_add_sync(0xFFFFFFFFu, ran);
+    if (lane == 0) {
+      if (part == 0) atomicAdd(&ctr->leaf_nodes, (unsigned long long)__popc(nodes));
+      if (all) atomicAdd(&ctr->leaves, (unsigned long long)all * (tc.alone_last ? tc.radix : 1u));
     }
-    if (ran) leaf_combos<NW>(tw, sdw, rtw, tc, slot, LeafShape<NW>::threads, dg, valid, c0, c1, lb);
   }
   // warp, then block minimum; one record update per block
 #pragma unroll
@@ -180,57 +230,58 @@ __global__ void __launch_bounds__(LeafShape<NW>::threads, LeafShape<NW>::min_blo
 
 size_t tree_node_words() { return (size_t)kNW; }
 
-cudaError_t launch_tree_root(const TablesW& tb, uint32_t* buf, uint32_t cap, cudaStream_t st) {
-  tree_root_kernel<<<1, 1, 0, st>>>(tb, buf, cap);
+cudaError_t launch_tree_bound(const uint32_t* ms, const uint8_t* fe, uint32_t n, uint32_t* bound, TreeCounters* ctr,
+                              cudaStream_t st) {
+  tree_bound_kernel<<<1, 1, 0, st>>>(ms, fe, n, bound, ctr);
   return cudaGetLastError();
 }
 
-cudaError_t launch_tree_expand(const TablesW& tb, const TreeConsts& tc, const uint32_t* src, uint32_t src_cap,
-                               uint32_t lo, uint32_t cnt, uint32_t d, uint32_t* dst, uint32_t dst_cap,
-                               unsigned long long* appended, unsigned long long base_total, const uint32_t* bound,
+cudaError_t launch_tree_start(const TablesW& tb, const TreeConsts& tc, uint32_t d0, TreeLevel dst, uint32_t cap,
+                              const uint32_t* bound, TreeCounters* ctr, cudaStream_t st) {
+  uint32_t combos = 1;
+  for (uint32_t i = 0; i < d0; ++i) combos *= tc.radix;
+  tree_start_kernel<<<(combos + kTreeThreads - 1) / kTreeThreads, kTreeThreads, 0, st>>>(tb, tc, d0, combos, dst, cap,
+                                                                                         bound, ctr);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_tree_expand(const TablesW& tb, const TreeConsts& tc, TreeLevel src, uint32_t pop,
+                               uint32_t most_nodes, uint32_t d, TreeLevel dst, uint32_t cap, const uint32_t* bound,
                                TreeCounters* ctr, cudaStream_t st) {
-  const uint64_t threads = (uint64_t)cnt * tc.radix;
+  const uint64_t threads = (uint64_t)(most_nodes < pop ? most_nodes : pop) * tc.radix;
   const unsigned grid = (unsigned)((threads + kTreeThreads - 1) / kTreeThreads);
-  tree_expand_kernel<<<grid, kTreeThreads, 0, st>>>(tb, tc, src, src_cap, lo, cnt, d, dst, dst_cap, appended, base_total, bound,
-                                                    ctr);
+  tree_expand_kernel<<<grid, kTreeThreads, 0, st>>>(tb, tc, src, pop, d, dst, cap, bound, ctr);
   return cudaGetLastError();
 }
 
 template <int NW>
-static cudaError_t leaf_launch(const TablesW& tb, const TreeConsts& tc, const uint32_t* src, uint32_t src_cap,
-                               uint32_t lo, uint32_t cnt, uint32_t parts, uint32_t chunk, unsigned grid,
-                               uint32_t* bound, BestRecord* best, TreeCounters* ctr, cudaStream_t st) {
+static cudaError_t leaf_launch(const TablesW& tb, const TreeConsts& tc, TreeLevel src, uint32_t cap,
+                               uint32_t most_nodes, uint32_t* bound, BestRecord* best, TreeCounters* ctr,
+                               cudaStream_t st) {
   static std::atomic<uint64_t> ready{0};
   const size_t smem = sizeof(uint32_t) * LaneWords<NW>::value * LeafShape<NW>::threads;
-  const cudaError_t e = allow_dyn_smem(tree_leaf_kernel<NW>, smem, &ready);
+  cudaError_t e = allow_dyn_smem(tree_leaf_kernel<NW>, smem, &ready);
+  int dev = 0, sms = 0;
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
   TablesT<NW> tw;
   host::build_window(tb, tc.W0, &tw);
-  const unsigned blocks = (unsigned)(((uint64_t)grid * kTreeWarps + LeafShape<NW>::warps - 1) / LeafShape<NW>::warps);
-  tree_leaf_kernel<NW><<<blocks, LeafShape<NW>::threads, smem, st>>>(tb, tw, tc, src, src_cap, lo, cnt, parts, chunk, bound, best,
-                                                         ctr);
+  // At most this many tasks (see the kernel), and a few waves of the GPU.
+  const uint64_t groups = (most_nodes + 31u) / 32u, tasks = kTreeLeafTasks + groups;
+  const uint64_t need = (tasks + LeafShape<NW>::warps - 1) / LeafShape<NW>::warps;
+  const uint64_t most = (uint64_t)sms * LeafShape<NW>::min_blocks * 8u;
+  tree_leaf_kernel<NW><<<(unsigned)(need < most ? need : most), LeafShape<NW>::threads, smem, st>>>(
+      tb, tw, tc, src, cap, bound, best, ctr);
   return cudaGetLastError();
 }
 
-cudaError_t launch_tree_leaf(const TablesW& tb, const TreeConsts& tc, const uint32_t* src, uint32_t src_cap,
-                             uint32_t lo, uint32_t cnt, uint32_t target_tasks, uint32_t* bound, BestRecord* best,
-                             TreeCounters* ctr, cudaStream_t st) {
-  // Split each group's combinations into parts so that about target_tasks
-  // warp tasks exist, each covering at least 16 combinations.
-  const uint32_t groups = (cnt + 31u) / 32u;
-  const uint32_t ncomb = tc.alone_last ? tc.combos / tc.radix : tc.combos;
-  uint32_t parts = (target_tasks + groups - 1u) / groups;
-  const uint32_t max_parts = (ncomb + 15u) / 16u;
-  if (parts > max_parts) parts = max_parts;
-  if (parts < 1u) parts = 1u;
-  const uint32_t chunk = (ncomb + parts - 1u) / parts;
-  parts = (ncomb + chunk - 1u) / chunk;
-  const uint64_t tasks = (uint64_t)groups * parts;
-  const unsigned grid = (unsigned)((tasks + kTreeWarps - 1) / kTreeWarps);
+cudaError_t launch_tree_leaf(const TablesW& tb, const TreeConsts& tc, TreeLevel src, uint32_t cap,
+                             uint32_t most_nodes, uint32_t* bound, BestRecord* best, TreeCounters* ctr,
+                             cudaStream_t st) {
   const uint32_t nw = tb.n - tc.W0;
-#define BF_TRY(NW)                                                                                           \
-  if (nw <= (uint32_t)NW)                                                                                    \
-    return leaf_launch<NW>(tb, tc, src, src_cap, lo, cnt, parts, chunk, grid, bound, best, ctr, st);
+#define BF_TRY(NW) \
+  if (nw <= (uint32_t)NW) return leaf_launch<NW>(tb, tc, src, cap, most_nodes, bound, best, ctr, st);
   BF_TREE_BUCKETS(BF_TRY)
 #undef BF_TRY
   return cudaErrorInvalidValue;

@@ -280,6 +280,86 @@ __device__ __forceinline__ bool expand_child(const TB& tb, const SD& sd, const u
   return !tc.prune || forward_bound<NT>(s, tb, tc, dg, assigned, ef, stride) <= bound;
 }
 
+// Node of the first d0 tools' modes `dg`, simulated from time 0 (s holds the
+// initial state): expand_child's test for d0 tools at once.
+template <int NT, typename TB, typename SD>
+__device__ __forceinline__ bool expand_start(const TB& tb, const SD& sd, const uint32_t* rt, const TreeConsts& tc,
+                                             State<NT>& s, Digits dg, uint32_t d0, uint32_t bound, uint32_t* ef,
+                                             uint32_t stride) {
+  if (dg.que & tb.big_mask) return false;
+  const uint32_t assigned = (1u << d0) - 1u;
+  if (run<NT>(s, tb, sd, rt, dg, tb.all_mask & ~assigned) != kRunStopped) return false;
+  return !tc.prune || forward_bound<NT>(s, tb, tc, dg, assigned, ef, stride) <= bound;
+}
+
+// The modes that each leaf tool may take in a mapping no worse than the bound,
+// as tool sets.
+struct LeafModes {
+  uint32_t cpu, now, que;
+};
+
+// The forward bound of leaf node j (forward_bound, over the leaf window, read
+// word by word from HBM) with the leaf tools open: false when every mapping
+// below the node is worse than `bound`; else *out has the modes of each leaf
+// tool in which it can end, with the longest minimum path after it, within the
+// bound (a GPU mode over the whole budget never starts).  A tool's earliest end
+// is the least over the modes it keeps.  `ef`: a column of the window's width
+// in shared memory.
+template <typename TB>
+__device__ __forceinline__ bool node_leaf_modes(const uint32_t* buf, uint32_t cap, uint32_t j, const TB& tb,
+                                                const TreeConsts& tc, Digits dg, uint32_t bound, uint32_t* ef,
+                                                uint32_t stride, LeafModes* out) {
+  const NodeSlots slot{buf + j, cap};
+  const uint32_t* t = buf + j + (size_t)(2 * kTreeSlots) * cap;
+  const uint32_t done = t[0], run_g = t[2 * (size_t)cap], T = t[4 * (size_t)cap], V = t[5 * (size_t)cap];
+  *out = LeafModes{0u, 0u, 0u};
+  uint64_t qsum = 0u;
+  for (uint32_t v = tc.W0; v < tc.n; ++v) {
+    const uint32_t bit = 1u << v;
+    if (done & bit) continue;
+    const uint32_t ec = slot.ec((int)v);
+    uint64_t fin = ~0ull;
+    if (ec != 0xFFFFFFFFu) {
+      fin = ec;
+    } else if (run_g & bit) {
+      const uint32_t r = slot.eg((int)v) - V;
+      const uint32_t left = (r >> 10) + ((r & 1023u) != 0u);
+      fin = (uint64_t)T + left;
+      if (dg.que & bit) qsum += left;
+    } else {
+      uint64_t start = T;
+      for (uint32_t m = tb.pred[v] & ~done; m; m &= m - 1u) {
+        const uint32_t e = ef[(__ffs(m) - 1u - tc.W0) * stride];
+        start = e > start ? e : start;
+      }
+      const uint32_t dc = tb.cpu[v], dn = tb.wnow[v] >> 10, dq = tb.wq[v] >> 10;
+      if (v < tc.leaf_level) {
+        fin = start + ((dg.now & bit) ? dn : (dg.que & bit) ? dq : dc);
+        if (dg.que & bit) qsum += dq;
+      } else {
+        const uint64_t after = start + tc.sdown[v];
+        const bool gpu = (tb.big_mask & bit) == 0u;
+        if (after + dc <= bound) {
+          out->cpu |= bit;
+          fin = start + dc;
+        }
+        if (gpu && after + dn <= bound) {
+          out->now |= bit;
+          fin = start + dn < fin ? start + dn : fin;
+        }
+        if (gpu && tc.radix == 3u && after + dq <= bound) {
+          out->que |= bit;
+          fin = start + dq < fin ? start + dq : fin;
+        }
+        if (fin == ~0ull) return false;
+      }
+    }
+    if (fin + tc.sdown[v] > bound) return false;
+    ef[(v - tc.W0) * stride] = (uint32_t)fin;
+  }
+  return T + qsum <= bound;
+}
+
 // Digits of leaf combination c (tools [L, n)), as masks shifted to tool L.
 __device__ __forceinline__ Digits leaf_digits(uint32_t c, uint32_t radix, uint32_t D, uint32_t L) {
   if (radix == 2u) return Digits{c << L, 0u};
@@ -324,46 +404,56 @@ struct LaneBest {
 // Simulate combinations [c0, c1) of the leaf node saved in `slot` (a lane's
 // shared-memory window state, stride `stride`) whose digits are `dg` (all
 // tools); tw/sdw/rtw are the window's tables.  `valid` false runs the loop
-// without work (lanes of a warp stay in lockstep).
+// without work (lanes of a warp stay in lockstep).  Only combinations of the
+// leaf tools' modes in `modes` are simulated (each lane passes over the others
+// before the warp simulates together), and a run past `bound` is given up;
+// returns how many were simulated.
 // With tc.alone_last, [c0, c1) are combinations of the leaf tools but the
 // last one: each is simulated until the last tool becomes ready (everything
 // else has ended then) and yields one makespan per mode of the last tool.
 template <int NW, typename TBW, typename SD>
-__device__ __forceinline__ void leaf_combos(const TBW& tw, const SD& sdw, const uint32_t* rtw, const TreeConsts& tc,
-                                            const uint32_t* slot, uint32_t stride, Digits dg, bool valid,
-                                            uint32_t c0, uint32_t c1, LaneBest& best) {
-  const uint32_t L = tc.leaf_level, W0 = tc.W0;
+__device__ __forceinline__ uint32_t leaf_combos(const TBW& tw, const SD& sdw, const uint32_t* rtw,
+                                                const TreeConsts& tc, const uint32_t* slot, uint32_t stride, Digits dg,
+                                                bool valid, uint32_t c0, uint32_t c1, LaneBest& best,
+                                                LeafModes modes = LeafModes{~0u, ~0u, ~0u},
+                                                uint32_t bound = 0xFFFFFFFFu) {
+  const uint32_t L = tc.leaf_level, W0 = tc.W0, D = tc.alone_last ? tc.D - 1u : tc.D;
   const Digits dgw{dg.now >> W0, dg.que >> W0};
-  if (tc.alone_last) {
-    const uint32_t last = tc.n - 1u, lastw = last - W0;
-    for (uint32_t c = c0; c < c1; ++c) {
-      if (!valid) continue;
-      const Digits dc = leaf_digits(c, tc.radix, tc.D - 1u, L - W0);
-      const Digits sim{dgw.now | dc.now, dgw.que | dc.que};
-      if (sim.que & tw.big_mask) continue;
-      State<NW> w;
-      load_lane(slot, stride, w);
-      if (run<NW>(w, tw, sdw, rtw, sim, 1u << lastw, 1u << lastw) != kRunStopped) continue;  // infeasible before it
-      const Digits full{dg.now | (dc.now << W0), dg.que | (dc.que << W0)};
+  const uint32_t leaf = D >= 32u ? ~0u : ((1u << D) - 1u);  // leaf tools, from bit 0
+  const LeafModes ok{modes.cpu >> L, modes.now >> L, modes.que >> L};
+  const uint32_t last = tc.n - 1u, lastw = last - W0;
+  uint32_t ran = 0u, c = valid ? c0 : c1;
+  Digits next = leaf_digits(c0, tc.radix, D, 0u);  // the modes of combination c
+  auto step = [&]() {
+    ++c;
+    if (tc.radix == 2u) next.now = c;
+    else increment(next);
+  };
+  for (;;) {
+    while (c < c1 && ((next.now & ~ok.now) | (next.que & ~ok.que) | (leaf & ~(next.now | next.que) & ~ok.cpu))) step();
+    if (c >= c1) break;
+    const Digits dc = next;
+    step();
+    const Digits sim{dgw.now | (dc.now << (L - W0)), dgw.que | (dc.que << (L - W0))};
+    if (sim.que & tw.big_mask) continue;
+    ++ran;
+    State<NW> w;
+    load_lane(slot, stride, w);
+    const uint32_t limit = best.ms < bound ? best.ms : bound;
+    const Digits full{dg.now | (dc.now << L), dg.que | (dc.que << L)};
+    if (tc.alone_last) {
+      if (run<NW>(w, tw, sdw, rtw, sim, 1u << lastw, 1u << lastw, limit) != kRunStopped) continue;  // infeasible before it
       for (uint32_t a = 0; a < tc.radix; ++a) {
         if (tc.alone[a] == kInfeasible) continue;
         best.offer(w.T + tc.alone[a],
                    Digits{full.now | (a == 1u ? 1u << last : 0u), full.que | (a == 2u ? 1u << last : 0u)},
                    tc.tie_pow3());
       }
+    } else if (run<NW>(w, tw, sdw, rtw, sim, 0u, 0u, limit) == kRunFinished) {
+      best.offer(w.T, full, tc.tie_pow3());
     }
-    return;
   }
-  for (uint32_t c = c0; c < c1; ++c) {
-    if (!valid) continue;
-    const Digits dc = leaf_digits(c, tc.radix, tc.D, L - W0);
-    const Digits sim{dgw.now | dc.now, dgw.que | dc.que};
-    if (sim.que & tw.big_mask) continue;
-    State<NW> w;
-    load_lane(slot, stride, w);
-    if (run<NW>(w, tw, sdw, rtw, sim, 0u) != kRunFinished) continue;
-    best.offer(w.T, Digits{dg.now | (dc.now << W0), dg.que | (dc.que << W0)}, tc.tie_pow3());
-  }
+  return ran;
 }
 
 namespace host {

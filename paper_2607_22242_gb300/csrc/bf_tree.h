@@ -19,20 +19,37 @@ struct __align__(16) BestRecord {
 
 // Device-side counters of one tree search.
 struct TreeCounters {
+  unsigned long long nodes;       // nodes appended to any level
   unsigned long long leaf_nodes;  // leaf-level nodes enumerated (counted by the warp task of their first chunk)
-  unsigned long long leaves;      // mappings simulated to the end by the leaf kernel
+  unsigned long long leaves;      // mappings simulated by the leaf kernel
+  uint32_t incumbent;             // the starting bound
   uint32_t error;                 // bit 0: a level buffer overflowed; bit 1: a best-record update gave up
-  uint32_t pad;
+};
+
+// A level of the search: its node buffer, and how many nodes have been
+// appended to it since it was last emptied (in device memory).
+struct TreeLevel {
+  uint32_t* buf;
+  uint32_t* count;
 };
 
 size_t tree_node_words();
-cudaError_t launch_tree_root(const TablesW& tb, uint32_t* buf, uint32_t cap, cudaStream_t st);
-cudaError_t launch_tree_expand(const TablesW& tb, const TreeConsts& tc, const uint32_t* src, uint32_t src_cap,
-                               uint32_t lo, uint32_t cnt, uint32_t d, uint32_t* dst, uint32_t dst_cap,
-                               unsigned long long* appended, unsigned long long base_total, const uint32_t* bound,
+// The starting bound: the least feasible of n candidates' makespans
+// (0xFFFFFFFF without one), to *bound and ctr->incumbent.
+cudaError_t launch_tree_bound(const uint32_t* ms, const uint8_t* fe, uint32_t n, uint32_t* bound, TreeCounters* ctr,
+                              cudaStream_t st);
+// Append the surviving nodes of the first d0 tools' modes to `dst` (level d0).
+cudaError_t launch_tree_start(const TablesW& tb, const TreeConsts& tc, uint32_t d0, TreeLevel dst, uint32_t cap,
+                              const uint32_t* bound, TreeCounters* ctr, cudaStream_t st);
+// Expand the last min(*src.count, pop) nodes of `src` (level d, at most
+// most_nodes of them) into `dst`; the counts are read on the device, so that
+// launches follow one another without the host.
+cudaError_t launch_tree_expand(const TablesW& tb, const TreeConsts& tc, TreeLevel src, uint32_t pop,
+                               uint32_t most_nodes, uint32_t d, TreeLevel dst, uint32_t cap, const uint32_t* bound,
                                TreeCounters* ctr, cudaStream_t st);
-cudaError_t launch_tree_leaf(const TablesW& tb, const TreeConsts& tc, const uint32_t* src, uint32_t src_cap,
-                             uint32_t lo, uint32_t cnt, uint32_t target_tasks, uint32_t* bound, BestRecord* best,
-                             TreeCounters* ctr, cudaStream_t st);
+// Enumerate the leaves of every node of `src`, the leaf level.
+cudaError_t launch_tree_leaf(const TablesW& tb, const TreeConsts& tc, TreeLevel src, uint32_t cap,
+                             uint32_t most_nodes, uint32_t* bound, BestRecord* best, TreeCounters* ctr,
+                             cudaStream_t st);
 
 }  // namespace bfk
