@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(kLtThreads, W ? kLtWideBlocksPerSm : kLtBlocks
   __syncthreads();
   MinKeySink sink;
   LtSharedT<NC>& Sref = S;
-  lt_lane<NC, W>(S, lt_rows_smem + threadIdx.x, blockDim.x,
+  lt_lane<NC, W, false, false, true>(S, lt_rows_smem + threadIdx.x, blockDim.x,
           [&Sref]() {
             const uint32_t r = atomicAdd(&Sref.root_next, 1u);
             return r < Sref.root_end ? r : 0xFFFFFFFFu;
@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(kLtThreads, W ? kLtWideBlocksPerSm : kLtBlocks
   for (uint32_t t = 0; t < S.rec.x; ++t) roots *= 3u;
   MinKeySink sink;
   LtSharedT<NC>& Sref = S;
-  lt_lane<NC, W, false, RANGE>(S, lt_rows_smem + threadIdx.x, blockDim.x,
+  lt_lane<NC, W, false, RANGE, !RANGE>(S, lt_rows_smem + threadIdx.x, blockDim.x,
           [&Sref, sync, static_roots, roots]() {
             const uint32_t r = atomicAdd(&Sref.root_next, 1u);
             if (r < Sref.root_end) return r;

@@ -439,19 +439,20 @@ inline void whole_space_tables(const bfk::Tables& t0, const bfk::Plan& p0, const
 }
 
 // Mappings a block of the lane-tree batch kernel aims to search (a 10-tool
-// scenario gets ceil(3^10 / 7381) = 9 blocks), and the fewest roots a block
-// hands out (two per lane of 256).  Many short blocks keep every SM busy to
-// the end of the launch: 4096 x 3^10 batch call, an earlier form of the
-// kernel, from 16.2 ms at one block per scenario (1024+ roots) to 14.8 ms at
-// 9 and 18.0 ms at 32 (128+); the current kernel at 7, 9, 12 and 16 blocks
-// per scenario 13.5, 13.4, 13.6 and 13.8 ms, at 9 blocks with 256+ roots
-// 13.4 ms.
-constexpr uint64_t kLtBlockMappings = 7381;
-constexpr uint64_t kLtMinRootsPerBlock = 512;
-// Blocks one scenario of a batch gets at most: with 512 roots per block this
+// scenario gets ceil(3^10 / 5000) = 12 blocks), and the fewest roots a block
+// hands out (one per lane of 256).  Many short blocks keep every SM busy to
+// the end of the launch.  Calls, ms, at 3700 / 5000 / 7381 / 15000 mappings
+// (256 roots): 4096 layered 10-tool scenarios 11.57 / 11.34 / 11.36 / 11.22, 200
+// of all shapes and 5 to 13 tools 1.81 / 1.85 / 2.04 / 2.21, 64 layered 10-tool
+// ones 0.55 / 0.57 / 0.62 / 0.80, 64 of 12 tools 2.18 / 2.16 / 2.15 / 2.29, 16 of
+// 14 tools 4.11 / 4.12 / 3.98 / 4.30; with 512 roots as many or up to 29 % more, with
+// 128 more on most.
+constexpr uint64_t kLtBlockMappings = 5000;
+constexpr uint64_t kLtMinRootsPerBlock = 256;
+// Blocks one scenario of a batch gets at most: with 256 roots per block this
 // keeps the roots of a 16-tool scenario at 12 tools (as its full search over
 // the whole GPU takes them) instead of 14, and a 20-tool one's at 12 instead
-// of 18 (472,000 blocks).  Scenarios of up to 14 tools stay below it.
+// of 18.  Scenarios of up to 14 tools stay below it.
 constexpr uint64_t kLtMaxBlocksPerScenario = 1024;
 
 // The levels of the lane-tree search of one scenario (n <= kLtMaxTools):
@@ -625,12 +626,12 @@ inline void lt_sample_events(const bfk::LaneTreeRecord& r, const uint8_t* mode, 
 // splits lanetree_levels allows, the one of least sampled cost -- a root
 // runs its mappings' steps up to ev[x], a level-1 job up to ev[y] from
 // there, a leaf to the end, and a job costs 0.3 steps more; jobs exist
-// only below checkpoints that were reached.  The cost grows by 0.6 / r for
-// r roots per lane (`lanes` lanes share them): the last roots of a search leave
-// lanes idle, the more so the fewer a lane runs.  Over all splits of 17 layered
-// and sparse DAGs of 12 to 17 tools, timed one by one, that choice is within 2 %
-// of the fastest split on average (1.21x at worst; without the second term
-// 1.21x for a 16-tool DAG, and roots far too few for the smaller ones).
+// only below checkpoints that were reached.  The cost grows by 0.2 / r for
+// r roots per lane (`lanes` lanes share them), or to 1 / r if that is more: the
+// last roots of a search leave lanes idle, the more so the fewer a lane runs.
+// Over all splits of 9 layered and sparse DAGs of 12 to 16 tools, timed one by
+// one, that choice is within 4 % of the fastest split on average (1.24x at
+// worst, a 13-tool DAG; with 0.6 / r 6 %).
 // Against levels from events alone with at least two roots per lane: 17-tool
 // layered DAG 9.1 -> 5.3 ms, 16-tool ones 1.59 -> 1.30 and 1.53 -> 1.53 ms,
 // 12-tool layered ones 112 -> 79 and 101 -> 70 us.
@@ -670,7 +671,8 @@ inline double lanetree_sampled_levels(const bfk::LaneTreeRecord& r, uint64_t min
       // kLtLevelSamples < 2^47.
       const uint64_t cost = 10u * (px * S[x] + py * (S[y] - S[x]) + pn * (S[n] - S[y])) +
                             3u * (px * kLtLevelSamples + (x < n ? py * A[x] : 0u) + (y < n ? pn * A[y] : 0u));
-      const uint64_t padded = cost + cost / px * (lanes * 6u / 10u);
+      const uint64_t fewer = cost / px * (lanes / 5u), thin = cost / px * lanes;
+      const uint64_t padded = cost + fewer > thin ? cost + fewer : thin;
       if (padded < best) {
         best = padded;
         *x_out = x;
