@@ -142,8 +142,8 @@ int search_tree_impl(const bf_scenario* scn_const, uint32_t space, uint32_t flag
   //    {256, 2048} nodes took 0.88 times the 8192 of a single dive on average
   //    ({256, 8192} 0.91, {1024, 8192} 0.92, {1024} 0.95, {64, 8192} 1.06).
   //    With these chains and the leaf modes (bf_tree.cuh node_leaf_modes) full
-  //    searches went from 2.30 to 1.28 ms (18 layered tools), 4.06 to 1.83 (20),
-  //    7.4 to 2.1 (24) and 6.4 to 2.1 ms (26).
+  //    searches went from 2.30 to 1.05 ms (18 layered tools), 4.06 to 1.90 (20),
+  //    7.4 to 2.1 (24) and 6.4 to 1.8 ms (26).
   static constexpr uint32_t kDives[] = {256, 2048};
   constexpr uint32_t kStart = 8192;
   // The whole search, not only each wait, is held to the wait limit.

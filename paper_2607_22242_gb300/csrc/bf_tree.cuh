@@ -401,59 +401,84 @@ struct LaneBest {
   }
 };
 
-// Simulate combinations [c0, c1) of the leaf node saved in `slot` (a lane's
-// shared-memory window state, stride `stride`) whose digits are `dg` (all
-// tools); tw/sdw/rtw are the window's tables.  `valid` false runs the loop
-// without work (lanes of a warp stay in lockstep).  Only combinations of the
-// leaf tools' modes in `modes` are simulated (each lane passes over the others
-// before the warp simulates together), and a run past `bound` is given up;
-// returns how many were simulated.
-// With tc.alone_last, [c0, c1) are combinations of the leaf tools but the
-// last one: each is simulated until the last tool becomes ready (everything
-// else has ended then) and yields one makespan per mode of the last tool.
+// Simulate one combination `dc` of the leaf tools' modes (bit 0: tool L) of the
+// leaf node saved in `slot` (a lane's shared-memory window state, stride
+// `stride`) whose digits are `dg` (all tools); tw/sdw/rtw are the window's
+// tables.  A run past `bound` or the best so far is given up; false when the
+// combination was not simulated (a queued tool larger than the budget).
+// With tc.alone_last, dc are modes of the leaf tools but the last one: the run
+// goes on until the last tool becomes ready (everything else has ended then)
+// and yields one makespan per mode of the last tool.
+template <int NW, typename TBW, typename SD>
+__device__ __forceinline__ bool leaf_run(const TBW& tw, const SD& sdw, const uint32_t* rtw, const TreeConsts& tc,
+                                         const uint32_t* slot, uint32_t stride, Digits dg, Digits dc, LaneBest& best,
+                                         uint32_t bound) {
+  const uint32_t L = tc.leaf_level, W0 = tc.W0, last = tc.n - 1u, lastw = last - W0;
+  const Digits full{dg.now | (dc.now << L), dg.que | (dc.que << L)};
+  const Digits sim{full.now >> W0, full.que >> W0};
+  if (sim.que & tw.big_mask) return false;
+  State<NW> w;
+  load_lane(slot, stride, w);
+  const uint32_t limit = best.ms < bound ? best.ms : bound;
+  if (tc.alone_last) {
+    if (run<NW>(w, tw, sdw, rtw, sim, 1u << lastw, 1u << lastw, limit) != kRunStopped) return true;  // infeasible before it
+    for (uint32_t a = 0; a < tc.radix; ++a) {
+      if (tc.alone[a] == kInfeasible) continue;
+      best.offer(w.T + tc.alone[a],
+                 Digits{full.now | (a == 1u ? 1u << last : 0u), full.que | (a == 2u ? 1u << last : 0u)},
+                 tc.tie_pow3());
+    }
+  } else if (run<NW>(w, tw, sdw, rtw, sim, 0u, 0u, limit) == kRunFinished) {
+    best.offer(w.T, full, tc.tie_pow3());
+  }
+  return true;
+}
+
+// Leaf tools whose modes a leaf run enumerates (all but a lone last one).
+__device__ __forceinline__ uint32_t leaf_tools(const TreeConsts& tc) { return tc.alone_last ? tc.D - 1u : tc.D; }
+
+// Combinations [c0, c1) of a leaf node's modes (leaf_run), all of them; returns
+// how many were simulated.  `valid` false runs the loop without work (lanes of a
+// warp stay in lockstep).
 template <int NW, typename TBW, typename SD>
 __device__ __forceinline__ uint32_t leaf_combos(const TBW& tw, const SD& sdw, const uint32_t* rtw,
                                                 const TreeConsts& tc, const uint32_t* slot, uint32_t stride, Digits dg,
-                                                bool valid, uint32_t c0, uint32_t c1, LaneBest& best,
-                                                LeafModes modes = LeafModes{~0u, ~0u, ~0u},
-                                                uint32_t bound = 0xFFFFFFFFu) {
-  const uint32_t L = tc.leaf_level, W0 = tc.W0, D = tc.alone_last ? tc.D - 1u : tc.D;
-  const Digits dgw{dg.now >> W0, dg.que >> W0};
-  const uint32_t leaf = D >= 32u ? ~0u : ((1u << D) - 1u);  // leaf tools, from bit 0
-  const LeafModes ok{modes.cpu >> L, modes.now >> L, modes.que >> L};
-  const uint32_t last = tc.n - 1u, lastw = last - W0;
-  uint32_t ran = 0u, c = valid ? c0 : c1;
-  Digits next = leaf_digits(c0, tc.radix, D, 0u);  // the modes of combination c
-  auto step = [&]() {
-    ++c;
-    if (tc.radix == 2u) next.now = c;
-    else increment(next);
-  };
-  for (;;) {
-    while (c < c1 && ((next.now & ~ok.now) | (next.que & ~ok.que) | (leaf & ~(next.now | next.que) & ~ok.cpu))) step();
-    if (c >= c1) break;
-    const Digits dc = next;
-    step();
-    const Digits sim{dgw.now | (dc.now << (L - W0)), dgw.que | (dc.que << (L - W0))};
-    if (sim.que & tw.big_mask) continue;
-    ++ran;
-    State<NW> w;
-    load_lane(slot, stride, w);
-    const uint32_t limit = best.ms < bound ? best.ms : bound;
-    const Digits full{dg.now | (dc.now << L), dg.que | (dc.que << L)};
-    if (tc.alone_last) {
-      if (run<NW>(w, tw, sdw, rtw, sim, 1u << lastw, 1u << lastw, limit) != kRunStopped) continue;  // infeasible before it
-      for (uint32_t a = 0; a < tc.radix; ++a) {
-        if (tc.alone[a] == kInfeasible) continue;
-        best.offer(w.T + tc.alone[a],
-                   Digits{full.now | (a == 1u ? 1u << last : 0u), full.que | (a == 2u ? 1u << last : 0u)},
-                   tc.tie_pow3());
-      }
-    } else if (run<NW>(w, tw, sdw, rtw, sim, 0u, 0u, limit) == kRunFinished) {
-      best.offer(w.T, full, tc.tie_pow3());
-    }
+                                                bool valid, uint32_t c0, uint32_t c1, LaneBest& best) {
+  uint32_t ran = 0u;
+  for (uint32_t c = c0; c < c1; ++c) {
+    if (!valid) continue;
+    ran += leaf_run<NW>(tw, sdw, rtw, tc, slot, stride, dg, leaf_digits(c, tc.radix, leaf_tools(tc), 0u), best,
+                        0xFFFFFFFFu) ? 1u : 0u;
   }
   return ran;
+}
+
+// Combinations of the leaf tools' modes that `modes` leaves (0 if a tool has
+// none), and the k-th of them: a mixed-radix number, the first leaf tool least
+// significant, each digit counting the modes its tool keeps.
+__device__ __forceinline__ uint32_t leaf_mode_combos(const LeafModes& modes, const TreeConsts& tc) {
+  uint32_t count = 1u;
+  for (uint32_t t = 0; t < leaf_tools(tc); ++t) {
+    const uint32_t bit = 1u << (tc.leaf_level + t);
+    count *= ((modes.cpu & bit) ? 1u : 0u) + ((modes.now & bit) ? 1u : 0u) + ((modes.que & bit) ? 1u : 0u);
+  }
+  return count;
+}
+
+__device__ __forceinline__ Digits leaf_mode_digits(const LeafModes& modes, const TreeConsts& tc, uint32_t k) {
+  Digits d{0u, 0u};
+  for (uint32_t t = 0; t < leaf_tools(tc); ++t) {
+    const uint32_t bit = 1u << (tc.leaf_level + t);
+    const bool c = modes.cpu & bit, n = modes.now & bit, q = modes.que & bit;
+    const uint32_t r = (c ? 1u : 0u) + (n ? 1u : 0u) + (q ? 1u : 0u);
+    const uint32_t next = r == 3u ? k / 3u : (r == 2u ? k >> 1 : k), j = k - next * r;
+    k = r == 1u ? k : next;
+    const uint32_t at = r == 1u ? 0u : j;  // the at-th mode the tool keeps
+    const uint32_t mode = at == 0u ? (c ? 0u : (n ? 1u : 2u)) : (at == 1u ? (c && n ? 1u : 2u) : 2u);
+    d.now |= mode == 1u ? 1u << t : 0u;
+    d.que |= mode == 2u ? 1u << t : 0u;
+  }
+  return d;
 }
 
 namespace host {
