@@ -269,8 +269,9 @@ def eval_mappings(h: Union[ScenarioHandle, Scenario], first: int, count: int, ou
                   out_feasible=None, stream=None):
     """Makespans (torch.int32 CUDA tensor holding u32 bit patterns) and feasibility
     flags (torch.uint8) of mappings [first, first+count).  Asynchronous on ``stream``;
-    the scenario's tables travel by value with the launch, so a temporary handle
-    may be released as soon as the call returns."""
+    the scenario's tables travel by value with the launch, and the memory of a
+    handle's segment tables is freed after the work that reads it, so a temporary
+    handle may be released as soon as the call returns."""
     import torch
     handle, owned = _handle(h)
     try:

@@ -467,14 +467,20 @@ bool segment_tables(const bf_scenario* scn, uint32_t** table) {
   uint32_t** slot = const_cast<uint32_t**>(&scn->d_table);
   *table = __atomic_load_n(slot, __ATOMIC_ACQUIRE);
   if (*table || scn->seg.entries == 0u) return true;
-  uint32_t* mine = nullptr;
-  if (lib_malloc(reinterpret_cast<void**>(&mine), sizeof(uint32_t) * scn->seg.entries) != cudaSuccess) {
+  // Another stream may be capturing: in this thread's relaxed mode the allocation
+  // neither fails nor ends that capture (no captured work uses the tables).
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  if (__atomic_compare_exchange_n(slot, table, mine, false, __ATOMIC_ACQ_REL, __ATOMIC_ACQUIRE)) *table = mine;
+  uint32_t* mine = nullptr;
+  const bool ok = lib_malloc(reinterpret_cast<void**>(&mine), sizeof(uint32_t) * scn->seg.entries) == cudaSuccess;
+  if (!ok) cudaGetLastError();
+  else if (__atomic_compare_exchange_n(slot, table, mine, false, __ATOMIC_ACQ_REL, __ATOMIC_ACQUIRE)) *table = mine;
   else cudaFree(mine);
-  return true;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  return ok;
 }
 
 // Whether a search of `count` mappings (not the whole space) of a scenario with
@@ -890,9 +896,7 @@ int bf_search_pruned(const bf_scenario* scn_const, uint64_t hint_index, bf_resul
 
 // A batch runs on the lane-tree batch kernel in up to three groups, one per
 // table form: up to kLtBatchTools tools, up to kLtNarrowTools, up to
-// kLtMaxTools (a 14-tool layered batch scenario ran on the prefix/mid/inner
-// batch kernel before; the no-alloc entry point still takes that kernel above
-// kLtBatchTools).  Batches of at least kBatchPipelineMin scenarios of the
+// kLtMaxTools.  Batches of at least kBatchPipelineMin scenarios of the
 // first group are pipelined: the first eighth of that group is built, copied
 // and launched on the caller's stream, and the rest of the batch is built
 // while that kernel runs and launched on a second stream (created for the

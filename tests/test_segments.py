@@ -159,6 +159,29 @@ def test_captured_evaluation_outlives_its_handle():
 
 
 @pytest.mark.gpu
+def test_first_evaluation_beside_a_capture():
+    """A handle's first evaluation (which allocates its tables) on one stream while another stream is being captured:
+    the capture goes on, and both give the right values."""
+    import torch
+    scn = S.config3()
+    first, count = 400_000_001, 1 << 18
+    x = torch.zeros(4, device="cuda")
+    want = bf.eval_mappings(scn, first, count)  # loads the kernels
+    ms = torch.zeros(count, dtype=torch.int32, device="cuda")
+    fe = torch.zeros(count, dtype=torch.uint8, device="cuda")
+    other = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with bf.create_scenario(scn) as h:
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            x.add_(1)
+            bf.eval_mappings(h, first, count, ms, fe, stream=other)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(ms, want[0]) and torch.equal(fe, want[1]) and (x == 1).all()
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("n,seg_max", [(2, 1), (9, 9), (20, 1), (32, 1), (32, 8), (27, 13)])
 def test_optimum_by_segments(n, seg_max):
     """Branch and bound over both spaces of scenarios cut by barriers, twice on one handle (the launch state resets
