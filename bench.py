@@ -47,12 +47,12 @@ OPS_PER_MAPPING = 2 * N_TOOLS * N_TOOLS
 INT_LANES_PER_SM = 128  # 4 SMSPs x 32 lanes: one thread instruction each per clock at full issue
 
 # Committed ncu summaries of the enumerating kernels, one per standard workload.
-PROFILES = {"config0": "search_kernel_config0_n8.md", "config1": "search_kernel_config1_n12.md",
+PROFILES = {"config0": "search_kernel_config0_n8.md", "config1": "lanetree_single_kernel_config1_n12.md",
             "config2": "lanetree_single_kernel_config2_n16.md", "config3": "search_kernel_config3_n19.md",
             "config4_batch": "lanetree_kernel_config4.md"}
-# Translation unit each summary's fingerprint covers (_build.kernel_fingerprint): the full search of
-# the 16-tool workload and the batch run the lane-tree kernels.
-PROFILE_UNITS = {"config2": "LANETREE_UNIT", "config4_batch": "LANETREE_UNIT"}
+# Translation unit each summary's fingerprint covers (_build.kernel_fingerprint): the full searches of
+# the 12- and 16-tool workloads and the batch run the lane-tree kernels.
+PROFILE_UNITS = {"config1": "LANETREE_UNIT", "config2": "LANETREE_UNIT", "config4_batch": "LANETREE_UNIT"}
 PROFILE_KEYS = ("source_fingerprint", "dram_bytes_per_launch", "thread_instructions_per_mapping", "issue_active",
                 "warp_efficiency", "kernel_ms")
 

@@ -1,8 +1,8 @@
-// bf_kernels.cu -- the three search kernels, compiled once per window width
+// bf_kernels.cu -- the enumerating kernels, compiled once per window width
 // (-DBF_NW=<slots>).  All integer ALU work: no tensor cores, and no HBM
 // streaming beyond the eval kernel's 5 bytes of output per mapping.
 //
-// Work decomposition (the same in all three kernels; see bfk::Plan).  A
+// Work decomposition (the same in every kernel; see bfk::Plan).  A
 // mapping index is idx = p + 3^P * (m + 3^M * i).  Each warp owns one prefix
 // p (the modes of tools [0, P)); its 32 lanes simulate that prefix together --
 // identical control flow -- until the first instant a tool >= P would become
@@ -19,8 +19,6 @@
 //            then warp shuffle-min -> block min -> one 64-bit atomicMin per
 //            block.  Ties go to the lowest index (the key's low word).  This is
 //            the brute-force oracle of §2.3 / §4.1 under the integer model.
-//   batch  : as search, for many independent scenarios in one launch; each
-//            block stages its scenario's tables and plan in shared memory.
 #include "bf_enum.cuh"
 #include "bf_launch.h"
 

@@ -10,7 +10,7 @@
 //                        survivors are appended to the next level's buffer
 //                        (one atomicAdd per warp on the level's count).
 //   tree_leaf_kernel   : one warp per 32 leaf-level nodes (one per lane) and a
-//                        chunk of the radix^D combinations of the last D tools,
+//                        chunk of the combinations of the last D tools' modes,
 //                        walked over the leaf window (tools from the
 //                        lowest one that can still be running at a leaf
 //                        checkpoint; compiled for 8..32 slots), without those
