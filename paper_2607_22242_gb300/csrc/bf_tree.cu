@@ -167,8 +167,15 @@ struct LeafShape {
 // 5.5 / 1.00 (dealt lanes leave the common path).  About kTreeLeafTasks tasks over
 // all nodes (each prepares its nodes anew; a quarter as many left lanes idle: 24
 // tools 2.6 against 2.1 ms), at least 16 combinations each, taken in turn by the
-// grid's warps.
+// grid's warps.  Few nodes are cut finer, down to 2 combinations a task, for about
+// kTreeLeafFill tasks: one warp for each place on the GPU (20 per SM), which
+// otherwise waits for a chain of 16 simulations on an eighth of them (the first
+// dive of an 18-tool search: 24 groups, 384 tasks, 390 us).  Full / binary space
+// before and after: 8 tools 0.18 -> 0.08 / 0.09 -> 0.08 ms, 16 layered tools 0.78
+// -> 0.63 / 0.38 -> 0.18, 18 tools 1.10 -> 0.86 / 0.43 -> 0.22, 20 tools 1.43 ->
+// 1.09 / 0.41 -> 0.23; 2 combinations for all of kTreeLeafTasks: 20 tools 1.55.
 constexpr uint32_t kTreeLeafTasks = 16384;
+constexpr uint32_t kTreeLeafFill = 3072;
 
 template <int NW>
 __global__ void __launch_bounds__(LeafShape<NW>::threads, LeafShape<NW>::min_blocks) tree_leaf_kernel(
@@ -183,7 +190,9 @@ __global__ void __launch_bounds__(LeafShape<NW>::threads, LeafShape<NW>::min_blo
   // With a lone last tool, combinations cover the leaf tools but the last
   // one, each standing for radix mappings.
   const uint32_t ncomb = tc.alone_last ? tc.combos / tc.radix : tc.combos;
-  const uint32_t want = max(1u, min((kTreeLeafTasks + groups - 1u) / max(groups, 1u), (ncomb + 15u) / 16u));
+  const uint32_t per = max(groups, 1u);
+  const uint32_t want = max(max(1u, min((kTreeLeafTasks + groups - 1u) / per, (ncomb + 15u) / 16u)),
+                            min(kTreeLeafFill / per, (ncomb + 1u) / 2u));
   const uint32_t chunk = (ncomb + want - 1u) / want, parts = (ncomb + chunk - 1u) / chunk;
   if (blockIdx.x * LeafShape<NW>::warps >= groups * parts) return;
   load_smem_tables(tw, sdw);

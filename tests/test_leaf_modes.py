@@ -11,9 +11,10 @@ THREADS = oracle.default_threads()
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("n", [1, 5, 6, 9, 13])
+@pytest.mark.parametrize("n", [1, 5, 6, 9, 10, 13])
 def test_optima_from_any_bound(n):
-    """No level above the leaves (5 tools and fewer), one start level only, start and expansions, and dives (13 tools):
+    """No level above the leaves (5 tools and fewer), one start level only (up to 8 levels
+    above the leaves; 1 to 243 leaf nodes, cut into parts of 2 combinations and more), start and expansions:
     hints at the optimum (the tightest bound that keeps it), at another mapping and none; small times, so that ties
     are frequent, tight budgets, late sources, a last tool that waits for all others."""
     rng = np.random.default_rng(n)
