@@ -135,15 +135,17 @@ int search_tree_impl(const bf_scenario* scn_const, uint32_t space, uint32_t flag
   //    leaf level) into the one after, and so on to the leaves; after the
   //    chain the host reads how many nodes each level has kept.  The levels
   //    below the one a chain starts from are empty.  The first chain starts
-  //    with every combination of the first d0 tools.  A large tree starts with
-  //    two dives, chains of kDives[i] nodes per level, whose leaves set the
-  //    bound; their other nodes are then dropped and the search starts over with
-  //    that bound.  Over 12 layered and sparse DAGs of 8 to 26 tools, dives of
+  //    with every combination of the first d0 tools.  A tree of more
+  //    leaf-level nodes than the start makes begins with two dives, chains of
+  //    kDives[i] nodes per level, whose leaves set the bound; their other nodes
+  //    are then dropped and the search starts over with that bound.  Over 12 layered and sparse DAGs of 8 to 26 tools, dives of
   //    {256, 2048} nodes took 0.88 times the 8192 of a single dive on average
   //    ({256, 8192} 0.91, {1024, 8192} 0.92, {1024} 0.95, {64, 8192} 1.06).
-  //    With these chains and the leaf modes (bf_tree.cuh node_leaf_modes) full
-  //    searches went from 2.30 to 1.05 ms (18 layered tools), 4.06 to 1.90 (20),
-  //    7.4 to 2.1 (24) and 6.4 to 1.8 ms (26).
+  //    Dives also pay below kPop leaf-level nodes (14 layered tools 0.62 -> 0.37 ms,
+  //    14 sparse ones 0.48 -> 0.36, the binary space of 24 tools 1.01 -> 0.73).
+  //    With these chains, the leaf modes (bf_tree.cuh node_leaf_modes) and the
+  //    leaf kernel's tasks full searches went from 2.30 to 0.86 ms (18 layered
+  //    tools), 4.06 to 1.4 (20), 7.4 to 1.7 (24) and 6.4 to 1.6 ms (26).
   static constexpr uint32_t kDives[] = {256, 2048};
   constexpr uint32_t kStart = 8192;
   // The whole search, not only each wait, is held to the wait limit.
@@ -155,7 +157,7 @@ int search_tree_impl(const bf_scenario* scn_const, uint32_t space, uint32_t flag
     start_nodes *= R;
     ++d0;
   }
-  for (uint32_t i = 0; i < tc.leaf_level && leaf_level_nodes <= kPop; ++i) leaf_level_nodes *= R;
+  for (uint32_t i = 0; i < tc.leaf_level && leaf_level_nodes <= kStart; ++i) leaf_level_nodes *= R;
   auto chain = [&](uint32_t from, uint64_t most, uint32_t pop) {  // most: nodes level `from` may hold
     for (uint32_t d = from; d < tc.leaf_level && e == cudaSuccess; ++d) {
       e = bfk::launch_tree_expand(tb, tc, tree_level(d), pop, (uint32_t)most, d, tree_level(d + 1), cap, &dv->bound,
@@ -173,7 +175,7 @@ int search_tree_impl(const bf_scenario* scn_const, uint32_t space, uint32_t flag
     ++launches;
   };
   start();
-  if (prune && leaf_level_nodes > kPop && e == cudaSuccess) {
+  if (prune && leaf_level_nodes > kStart && e == cudaSuccess) {
     for (const uint32_t pop : kDives) {
       if (e == cudaSuccess) chain(d0, start_nodes, pop);
       if (e == cudaSuccess) e = cudaMemsetAsync(dv->count, 0, sizeof dv->count, st);

@@ -11,14 +11,14 @@ THREADS = oracle.default_threads()
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("n", [1, 5, 6, 9, 10, 13])
+@pytest.mark.parametrize("n", [1, 5, 6, 9, 10, 13, 14])
 def test_optima_from_any_bound(n):
-    """No level above the leaves (5 tools and fewer), one start level only (up to 8 levels
-    above the leaves; 1 to 243 leaf nodes, cut into parts of 2 combinations and more), start and expansions:
-    hints at the optimum (the tightest bound that keeps it), at another mapping and none; small times, so that ties
-    are frequent, tight budgets, late sources, a last tool that waits for all others."""
+    """No level above the leaves (5 tools and fewer), one start level only (1 to 243 leaf nodes, cut into parts of 2
+    combinations and more), start and expansions, and dives (14 tools): hints at the optimum (the tightest bound that
+    keeps it), at another mapping and none; small times, so that ties are frequent, tight budgets, late sources, a last
+    tool that waits for all others."""
     rng = np.random.default_rng(n)
-    for t in range(8 if n < 13 else 4):
+    for t in range(8 if n < 13 else 4 if n < 14 else 2):
         base = S.random_small(rng, n, edge_p=float(rng.choice([0.1, 0.4])), tight=bool(t % 3), contention=bool(t % 4),
                               max_time=int(rng.choice([3, 9, 60])))
         pred = list(base.pred_mask)
