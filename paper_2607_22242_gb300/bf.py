@@ -325,8 +325,10 @@ def _batch_call(fn, scns: Sequence[Scenario], stream, packed=None) -> List[Resul
         return []
     import numpy as np
     arr = np.ctypeslib.as_array(results)  # one structured view instead of per-field ctypes reads
-    modes = arr["mode"][:, :max(sc.n for sc in scns)].tolist()
-    return [Result(i, m, bool(f), md[:sc.n]) for i, m, f, md, sc in
+    width = max(sc.n for sc in scns)
+    modes = arr["mode"][:, :width].tolist()
+    # Rows of full width are taken as they are: a copy of each is one more object per result for the collector.
+    return [Result(i, m, bool(f), md if sc.n == width else md[:sc.n]) for i, m, f, md, sc in
             zip(arr["index"].tolist(), arr["makespan_us"].tolist(), arr["feasible"].tolist(), modes, scns)]
 
 
