@@ -419,7 +419,7 @@ __device__ __forceinline__ void lt_lane(const LtSharedT<NC>& S, uint32_t* rows, 
   uint32_t end1 = cnt1;   // this lane's level-1 combinations end here
   bool idle = false;      // SHARE: no root was left, and no work to share
   for (;;) {
-#ifdef __CUDACC__
+#if defined(__CUDACC__) || defined(BF_HOST_WARP)  // (or a host build with the warp's collectives)
     if constexpr (SHARE) {
       const uint32_t idlers = __ballot_sync(0xFFFFFFFFu, idle);
       if (idlers) {
@@ -440,6 +440,7 @@ __device__ __forceinline__ void lt_lane(const LtSharedT<NC>& S, uint32_t* rows, 
           const uint32_t t_mid = __shfl_sync(0xFFFFFFFFu, mid, from), t_end = __shfl_sync(0xFFFFFFFFu, end1, from);
           const uint32_t t_now = __shfl_sync(0xFFFFFFFFu, now, from), t_que = __shfl_sync(0xFFFFFFFFu, que, from);
           const uint32_t t_idx0 = __shfl_sync(0xFFFFFFFFu, idx0, from);
+          __syncwarp();  // the donors' rows were written in earlier passes: votes and shuffles order no memory
           if (takes) {
             const uint32_t* src = rows + (int)(from - lane);
             for (uint32_t w = 0; w < n + SW; ++w) rows[w * stride] = src[w * stride];
@@ -453,7 +454,7 @@ __device__ __forceinline__ void lt_lane(const LtSharedT<NC>& S, uint32_t* rows, 
             idle = false;
           }
           if (gives) end1 = mid;
-          __syncwarp();
+          __syncwarp();  // the copies are made before a donor writes its rows again
         }
       }
       if (idle) continue;

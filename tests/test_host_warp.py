@@ -1,0 +1,48 @@
+"""Device code whose lanes read each other's shared memory, on a CPU warp without memory ordering between
+__syncwarps (tests/host_warp.h), against the oracle (no GPU)."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2607_22242_gb300 import bf
+from paper_2607_22242_gb300 import scenarios as S
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+THREADS = oracle.default_threads()
+
+
+@pytest.fixture(scope="module")
+def warp(tmp_path_factory):
+    out = str(tmp_path_factory.mktemp("warp") / "host_warp.so")
+    subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-Wno-unknown-pragmas", "-I",
+                    os.path.join(HERE, "..", "include"), "-o", out, os.path.join(HERE, "host_warp.cpp")], check=True)
+    lib = ctypes.CDLL(out)
+    lib.host_lanetree_warp.argtypes = [ctypes.POINTER(bf.Desc), ctypes.c_uint32, ctypes.c_uint32, ctypes.c_int,
+                                       ctypes.c_void_p, ctypes.c_void_p]
+    lib.host_lanetree_warp.restype = ctypes.c_int
+    return lib
+
+
+@pytest.mark.parametrize("n,x,y", [(5, 1, 3), (7, 1, 4), (7, 2, 4), (8, 3, 7), (8, 4, 8)])
+@pytest.mark.parametrize("wide", [False, True])
+def test_lanes_take_over_combinations(warp, n, x, y, wide):
+    """Fewer roots than lanes, and a few more (three levels and two): every feasible mapping reported once with the
+    oracle's makespan, most of them by lanes that took over another's combinations."""
+    rng = np.random.default_rng(n * 100 + x * 10 + y)
+    shared = np.zeros(1, np.uint32)
+    taken = 0
+    for t in range(4):
+        scn = S.random_small(rng, n, edge_p=float(rng.choice([0.1, 0.4])), tight=bool(t % 2), contention=True,
+                             max_time=int(rng.choice([5, 40])))
+        got = np.zeros(3 ** n, np.uint32)
+        assert warp.host_lanetree_warp(ctypes.byref(bf.to_desc(scn)), x, y, int(wide), got.ctypes.data,
+                                       shared.ctypes.data) == 0
+        want, _ = oracle.eval_range(scn, 0, 3 ** n, THREADS)
+        bad = np.flatnonzero(got.astype(np.uint64) != want)
+        assert bad.size == 0, (t, bad.size, int(bad[0]))
+        taken += int(shared[0])
+    assert taken > 0
