@@ -33,10 +33,6 @@ constexpr int kTreeThreads = 256;
 constexpr int kTreeWarps = kTreeThreads / 32;
 constexpr int kNW = NodeWords<kTreeSlots>::value;
 
-__device__ __forceinline__ uint32_t read_bound(const uint32_t* bound) {
-  return *reinterpret_cast<const volatile uint32_t*>(bound);
-}
-
 __device__ __forceinline__ uint32_t read_count(const uint32_t* count) {
   return *reinterpret_cast<const volatile uint32_t*>(count);
 }
@@ -153,18 +149,7 @@ struct LeafShape {
   static constexpr int min_blocks = NW <= 12 ? 4 : NW <= 16 ? 6 : NW <= 24 ? 5 : 4;
 };
 
-// A warp task is a part of the mappings below 32 nodes, one node's modes and
-// state prepared by each lane.  Unpruned, the lanes walk the combinations of
-// their own nodes in lockstep, which keeps them on one path (99 %).  Pruned, the
-// combinations that the bound leaves differ from node to node (a handful of 243
-// in some, none in most): while the nodes keep about as many each, every lane
-// walks its own node's; else (fewer than 12 times the fullest node's in all) they
-// are dealt to the lanes one by one over all 32 nodes, a lane resuming the state
-// of whichever node its combination belongs to.  A 24-tool layered DAG had 3.3 of
-// 32 lanes at work with every lane on its own node.  Full searches, own nodes only
-// / dealt only / by this rule: 14 layered tools 0.87 / 0.77 / 0.60 ms, 18 tools
-// 1.28 / 1.36 / 1.05, 26 tools 2.13 / 1.92 / 1.80; binary space of 24 tools 1.20 /
-// 5.5 / 1.00 (dealt lanes leave the common path).  About kTreeLeafTasks tasks over
+// The tasks of the leaf kernel (leaf_task). About kTreeLeafTasks tasks over
 // all nodes (each prepares its nodes anew; a quarter as many left lanes idle: 24
 // tools 2.6 against 2.1 ms), at least 16 combinations each, taken in turn by the
 // grid's warps.  Few nodes are cut finer, down to 2 combinations a task, for about
@@ -199,71 +184,16 @@ __global__ void __launch_bounds__(LeafShape<NW>::threads, LeafShape<NW>::min_blo
   fill_ready_table<NW>(tw, rtw);
   __syncthreads();
   LaneBest lb;
-  constexpr uint32_t stride = LeafShape<NW>::threads;
   uint32_t* const slot = lane_state + threadIdx.x;
   for (uint32_t task = blockIdx.x * LeafShape<NW>::warps + warp; task < groups * parts;
        task += gridDim.x * LeafShape<NW>::warps) {
-    const uint32_t g = task / parts, part = task - g * parts, j = g * 32u + lane;
-    bool valid = j < cnt;
-    Digits dg{0u, 0u};
-    LeafModes modes{0u, 0u, 0u};
-    uint32_t limit = tc.prune ? read_bound(bound) : kInfeasible;
-    __syncwarp();  // the other lanes are done with this lane's state
-    if (valid) {
-      const uint32_t* t = src.buf + j + (size_t)(2 * kTreeSlots) * cap;
-      dg = Digits{t[9 * (size_t)cap], t[10 * (size_t)cap]};
-      // The incumbent may have improved since this node was bounded; only modes
-      // within it are enumerated.
-      if (tc.prune) valid = node_leaf_modes(src.buf, cap, j, tb, tc, dg, limit, slot, stride, &modes);
-      if (valid) node_to_window<NW>(src.buf, cap, j, tc.W0, tw.n, slot, stride);
-    }
-    const uint32_t nodes = __ballot_sync(0xFFFFFFFFu, valid);
+    uint32_t nodes;
+    const uint32_t ran = leaf_task<NW, LeafShape<NW>::threads>(tb, tw, sdw, rtw, tc, src.buf, cap, cnt, task / parts,
+                                                               task % parts, parts, chunk, bound, slot, lb, &nodes);
     if (nodes == 0u) continue;
-    uint32_t ran = 0u;
-    uint32_t upto = valid && tc.prune ? leaf_mode_combos(modes, tc) : 0u;  // combinations of lanes 0 .. this one
-    const uint32_t most = __reduce_max_sync(0xFFFFFFFFu, upto), sum = __reduce_add_sync(0xFFFFFFFFu, upto);
-    if (tc.prune && sum < most * 12u) {
-#pragma unroll
-      for (uint32_t o = 1; o < 32u; o <<= 1) {
-        const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, upto, o);
-        if (lane >= o) upto += v;
-      }
-      const uint32_t total = __shfl_sync(0xFFFFFFFFu, upto, 31);
-      const uint32_t q0 = (uint32_t)((uint64_t)total * part / parts), q1 = (uint32_t)((uint64_t)total * (part + 1u) / parts);
-      for (uint32_t base = q0; base < q1; base += 32u) {
-        const uint32_t q = min(base + lane, q1 - 1u);
-        uint32_t i = 0u;  // the node whose combinations include the q-th: the first lane with upto > q
-#pragma unroll
-        for (uint32_t step = 16; step; step >>= 1)
-          if (__shfl_sync(0xFFFFFFFFu, upto, i + step - 1u) <= q) i += step;
-        const uint32_t before = __shfl_sync(0xFFFFFFFFu, upto, i ? i - 1u : 0u);
-        const LeafModes m{__shfl_sync(0xFFFFFFFFu, modes.cpu, i), __shfl_sync(0xFFFFFFFFu, modes.now, i),
-                          __shfl_sync(0xFFFFFFFFu, modes.que, i)};
-        const Digits d{__shfl_sync(0xFFFFFFFFu, dg.now, i), __shfl_sync(0xFFFFFFFFu, dg.que, i)};
-        if (base + lane < q1) {
-          limit = min(limit, read_bound(bound));
-          const Digits dc = leaf_mode_digits(m, tc, q - (i ? before : 0u));
-          ran += leaf_run<NW>(tw, sdw, rtw, tc, slot + (int)(i - lane), stride, d, dc, lb, limit) ? 1u : 0u;
-        }
-        __syncwarp();
-      }
-    } else if (tc.prune) {
-      const uint32_t q0 = upto * part / parts, q1 = upto * (part + 1u) / parts;
-      const uint32_t rounds = __reduce_max_sync(0xFFFFFFFFu, q1 - q0);
-      for (uint32_t k = 0; k < rounds; ++k) {
-        if (q0 + k < q1) {
-          limit = min(limit, read_bound(bound));
-          ran += leaf_run<NW>(tw, sdw, rtw, tc, slot, stride, dg, leaf_mode_digits(modes, tc, q0 + k), lb, limit) ? 1u : 0u;
-        }
-        __syncwarp();
-      }
-    } else {
-      const uint32_t c0 = part * chunk, c1 = min(c0 + chunk, ncomb);
-      ran = leaf_combos<NW>(tw, sdw, rtw, tc, slot, stride, dg, valid, c0, c1, lb);
-    }
     const uint32_t all = __reduce_add_sync(0xFFFFFFFFu, ran);
     if (lane == 0) {
-      if (part == 0) atomicAdd(&ctr->leaf_nodes, (unsigned long long)__popc(nodes));
+      if (task % parts == 0) atomicAdd(&ctr->leaf_nodes, (unsigned long long)__popc(nodes));
       if (all) atomicAdd(&ctr->leaves, (unsigned long long)all * (tc.alone_last ? tc.radix : 1u));
     }
   }

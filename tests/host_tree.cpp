@@ -22,10 +22,8 @@ static inline int __clz(unsigned x) { return x ? __builtin_clz(x) : 32; }
 static inline unsigned long long __umul64hi(unsigned long long a, unsigned long long b) {
   return (unsigned long long)(((unsigned __int128)a * b) >> 64);
 }
-struct HostDim {
-  unsigned x;
-};
-static HostDim threadIdx{0}, blockDim{1};
+
+#include "host_warp.h"
 
 #include "../paper_2607_22242_gb300/csrc/bf_tree.cuh"
 

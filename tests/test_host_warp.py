@@ -24,6 +24,9 @@ def warp(tmp_path_factory):
     lib.host_lanetree_warp.argtypes = [ctypes.POINTER(bf.Desc), ctypes.c_uint32, ctypes.c_uint32, ctypes.c_int,
                                        ctypes.c_void_p, ctypes.c_void_p]
     lib.host_lanetree_warp.restype = ctypes.c_int
+    lib.host_leaf_warps.argtypes = [ctypes.POINTER(bf.Desc), ctypes.c_uint32, ctypes.c_int, ctypes.c_uint32,
+                                    ctypes.c_uint32, ctypes.c_void_p, ctypes.c_void_p]
+    lib.host_leaf_warps.restype = ctypes.c_int
     return lib
 
 
@@ -46,3 +49,28 @@ def test_lanes_take_over_combinations(warp, n, x, y, wide):
         assert bad.size == 0, (t, bad.size, int(bad[0]))
         taken += int(shared[0])
     assert taken > 0
+
+
+def _leaves(warp, scn, space, start, bounds, prune=True):
+    """((index, makespan), mappings simulated, nodes of the first tasks, leaf nodes) of the leaf tasks."""
+    out, b = np.zeros(5, np.uint64), np.array(bounds, np.uint32)
+    assert warp.host_leaf_warps(ctypes.byref(bf.to_desc(scn)), space, int(prune), start, b.size, b.ctypes.data,
+                                out.ctypes.data) == 0
+    ms, idx = int(out[0]), int(out[1])
+    return (idx, ms) if ms != 2 ** 64 - 1 else (-1, 0xFFFFFFFF), int(out[2]), int(out[3]), int(out[4])
+
+
+@pytest.mark.parametrize("n", [6, 8, 10])
+@pytest.mark.parametrize("parts", [1, 3, 16])
+def test_leaf_tasks_share_nodes(warp, n, parts):
+    """Leaf groups from no bound (every lane on its own node), from just above the optimum and at it (few
+    combinations, dealt over the lanes, which read one another's states), and unpruned: the oracle's optimum."""
+    rng = np.random.default_rng(n)
+    for t in range(3):
+        scn = S.random_small(rng, n, edge_p=0.3, tight=bool(t % 2), contention=True, max_time=(9, 60, 500)[t])
+        for space, want in ((3, oracle.search(scn, THREADS)), (2, oracle.search_binary(scn, THREADS))):
+            for start in (0xFFFFFFFF, want[1] + want[1] // 10, want[1]):
+                got = _leaves(warp, scn, space, start, [start] * parts)
+                assert got[0] == want, (t, space, start, got, want)
+            if n <= 8:
+                assert _leaves(warp, scn, space, 0xFFFFFFFF, [0xFFFFFFFF] * parts, prune=False)[0] == want
