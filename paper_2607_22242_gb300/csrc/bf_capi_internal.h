@@ -28,8 +28,7 @@ struct bf_scratch {
   uint32_t survivors;   // pruned search: number of surviving prefixes
   uint32_t pruned_bound;  // pruned search: the incumbent's makespan (set with survivors)
   bfk::BestRecord best;      // tree search: best (makespan, index) so far
-  uint32_t bound;            // tree search: makespan bound for pruning
-  uint32_t pad2;
+  bfk::TreeBounds bounds;    // tree search: makespan bounds for pruning
   bfk::TreeCounters ctr;     // tree search: counters and error bits
   uint32_t count[BF_MAX_TOOLS + 1];  // tree search: nodes of each level
   uint64_t idx[BF_MAX_PROBES];

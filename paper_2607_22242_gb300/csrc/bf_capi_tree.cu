@@ -96,7 +96,7 @@ int search_tree_impl(const bf_scenario* scn_const, uint32_t space, uint32_t flag
   //    written again before the first wait below).
   h->best.ms = ~0ull;
   h->best.idx = ~0ull;
-  h->bound = 0xFFFFFFFFu;
+  h->bounds.live = h->bounds.leaf = 0xFFFFFFFFu;
   std::memset(&h->ctr, 0, sizeof h->ctr);
   h->ctr.incumbent = 0xFFFFFFFFu;
   std::memset(h->count, 0, sizeof h->count);
@@ -124,7 +124,7 @@ int search_tree_impl(const bf_scenario* scn_const, uint32_t space, uint32_t flag
     h->idx[nc++] = fast;
     if (R == 3) h->idx[nc++] = 2 * now;
     e = launch_list(scn, scn->d_host_scratch->idx, nc, dv->ms, dv->fe, st);
-    if (e == cudaSuccess) e = bfk::launch_tree_bound(dv->ms, dv->fe, nc, &dv->bound, &dv->ctr, st);
+    if (e == cudaSuccess) e = bfk::launch_tree_bound(dv->ms, dv->fe, nc, &dv->bounds, &dv->ctr, st);
     launches += 2;
   }
   if (e != cudaSuccess) return cuda_fail(e, who);
@@ -160,18 +160,18 @@ int search_tree_impl(const bf_scenario* scn_const, uint32_t space, uint32_t flag
   for (uint32_t i = 0; i < tc.leaf_level && leaf_level_nodes <= kStart; ++i) leaf_level_nodes *= R;
   auto chain = [&](uint32_t from, uint64_t most, uint32_t pop) {  // most: nodes level `from` may hold
     for (uint32_t d = from; d < tc.leaf_level && e == cudaSuccess; ++d) {
-      e = bfk::launch_tree_expand(tb, tc, tree_level(d), pop, (uint32_t)most, d, tree_level(d + 1), cap, &dv->bound,
+      e = bfk::launch_tree_expand(tb, tc, tree_level(d), pop, (uint32_t)most, d, tree_level(d + 1), cap, &dv->bounds,
                                   &dv->ctr, st);
       most = (most < pop ? most : pop) * R;
       ++launches;
     }
     if (e == cudaSuccess)
-      e = bfk::launch_tree_leaf(tb, tc, tree_level(tc.leaf_level), cap, (uint32_t)most, &dv->bound, &dv->best,
+      e = bfk::launch_tree_leaf(tb, tc, tree_level(tc.leaf_level), cap, (uint32_t)most, &dv->bounds, &dv->best,
                                 &dv->ctr, st);
     ++launches;
   };
   auto start = [&]() {
-    e = bfk::launch_tree_start(tb, tc, d0, tree_level(d0), cap, &dv->bound, &dv->ctr, st);
+    e = bfk::launch_tree_start(tb, tc, d0, tree_level(d0), cap, &dv->bounds, &dv->ctr, st);
     ++launches;
   };
   start();

@@ -37,13 +37,18 @@ __device__ __forceinline__ uint32_t read_count(const uint32_t* count) {
   return *reinterpret_cast<const volatile uint32_t*>(count);
 }
 
-__global__ void tree_bound_kernel(const uint32_t* ms, const uint8_t* fe, uint32_t n, uint32_t* bound,
+__global__ void tree_bound_kernel(const uint32_t* ms, const uint8_t* fe, uint32_t n, TreeBounds* bounds,
                                   TreeCounters* ctr) {
   uint32_t b = kInfeasible;
   for (uint32_t j = 0; j < n; ++j)
     if (fe[j] == 1u && ms[j] < b) b = ms[j];
-  *bound = b;
+  bounds->live = b;
   ctr->incumbent = b;
+}
+
+// The bound of the coming leaf launch (TreeBounds::leaf).
+__device__ __forceinline__ void note_leaf_bound(TreeBounds* bounds) {
+  if (blockIdx.x == 0u && threadIdx.x == 0u) bounds->leaf = read_bound(&bounds->live);
 }
 
 // Append this lane's node (if it keeps one) to a level: a slot per lane from
@@ -70,10 +75,11 @@ __device__ __forceinline__ void append_node(bool keep, const State<kTreeSlots>& 
 
 __global__ void __launch_bounds__(kTreeThreads, 2) tree_start_kernel(
     const __grid_constant__ TablesW tb, const __grid_constant__ TreeConsts tc, uint32_t d0, uint32_t combos,
-    TreeLevel dst, uint32_t cap, const uint32_t* bound, TreeCounters* ctr) {
+    TreeLevel dst, uint32_t cap, TreeBounds* bounds, TreeCounters* ctr) {
   __shared__ SmemTablesW sd;
   __shared__ uint32_t rt[ReadyTable<kTreeSlots>::size];
   __shared__ uint32_t ef[kTreeSlots * kTreeThreads];  // forward_bound scratch, [tool][thread]
+  note_leaf_bound(bounds);
   load_smem_tables(tb, sd);
   fill_ready_table<kTreeSlots>(tb, rt);
   __syncthreads();
@@ -84,17 +90,18 @@ __global__ void __launch_bounds__(kTreeThreads, 2) tree_start_kernel(
   if (p < combos) {
     dg = leaf_digits(p, tc.radix, d0, 0u);
     init_state(s, tb.all_mask);
-    keep = expand_start<kTreeSlots>(tb, sd, rt, tc, s, dg, d0, read_bound(bound), ef + threadIdx.x, kTreeThreads);
+    keep = expand_start<kTreeSlots>(tb, sd, rt, tc, s, dg, d0, read_bound(&bounds->live), ef + threadIdx.x, kTreeThreads);
   }
   append_node(keep, s, dg, dst, cap, ctr);
 }
 
 __global__ void __launch_bounds__(kTreeThreads, 2) tree_expand_kernel(
     const __grid_constant__ TablesW tb, const __grid_constant__ TreeConsts tc, TreeLevel src, uint32_t pop, uint32_t d,
-    TreeLevel dst, uint32_t cap, const uint32_t* bound, TreeCounters* ctr) {
+    TreeLevel dst, uint32_t cap, TreeBounds* bounds, TreeCounters* ctr) {
   __shared__ SmemTablesW sd;
   __shared__ uint32_t rt[ReadyTable<kTreeSlots>::size];
   __shared__ uint32_t ef[kTreeSlots * kTreeThreads];  // forward_bound scratch, [tool][thread]
+  note_leaf_bound(bounds);
   // Thread t: mode a = t / cnt of tool d for parent lo + t % cnt, so that a
   // warp's lanes hold neighbouring parents with the same new mode.
   const uint32_t size = read_count(src.count), cnt = min(size, pop), lo = size - cnt;
@@ -109,7 +116,7 @@ __global__ void __launch_bounds__(kTreeThreads, 2) tree_expand_kernel(
   Digits dg{0u, 0u};
   if (a < tc.radix) {
     load_node(src.buf, cap, lo + j, s, dg);
-    keep = expand_child<kTreeSlots>(tb, sd, rt, tc, s, dg, d, a, read_bound(bound), ef + threadIdx.x, kTreeThreads);
+    keep = expand_child<kTreeSlots>(tb, sd, rt, tc, s, dg, d, a, read_bound(&bounds->live), ef + threadIdx.x, kTreeThreads);
   }
   append_node(keep, s, dg, dst, cap, ctr);
 }
@@ -165,7 +172,7 @@ constexpr uint32_t kTreeLeafFill = 3072;
 template <int NW>
 __global__ void __launch_bounds__(LeafShape<NW>::threads, LeafShape<NW>::min_blocks) tree_leaf_kernel(
     const __grid_constant__ TablesW tb, const __grid_constant__ TablesT<NW> tw, const __grid_constant__ TreeConsts tc,
-    TreeLevel src, uint32_t cap, uint32_t* bound, BestRecord* best, TreeCounters* ctr) {
+    TreeLevel src, uint32_t cap, TreeBounds* bounds, BestRecord* best, TreeCounters* ctr) {
   extern __shared__ uint32_t lane_state[];
   __shared__ SmemTablesT<NW> sdw;
   __shared__ uint32_t rtw[ReadyTable<NW>::size];
@@ -189,7 +196,7 @@ __global__ void __launch_bounds__(LeafShape<NW>::threads, LeafShape<NW>::min_blo
        task += gridDim.x * LeafShape<NW>::warps) {
     uint32_t nodes;
     const uint32_t ran = leaf_task<NW, LeafShape<NW>::threads>(tb, tw, sdw, rtw, tc, src.buf, cap, cnt, task / parts,
-                                                               task % parts, parts, chunk, bound, slot, lb, &nodes);
+                                                               task % parts, parts, chunk, bounds, slot, lb, &nodes);
     if (nodes == 0u) continue;
     const uint32_t all = __reduce_add_sync(0xFFFFFFFFu, ran);
     if (lane == 0) {
@@ -213,7 +220,7 @@ __global__ void __launch_bounds__(LeafShape<NW>::threads, LeafShape<NW>::min_blo
     LaneBest b;
     for (int w = 0; w < LeafShape<NW>::warps; ++w) b.offer(wb_ms[w], Digits{wb_now[w], wb_que[w]}, tc.tie_pow3());
     if (b.ms != kInfeasible) {
-      atomicMin(bound, b.ms);
+      atomicMin(&bounds->live, b.ms);
       best_min(best, b.ms, index_of(b.dg, tc.pow3), ctr);
     }
   }
@@ -223,33 +230,33 @@ __global__ void __launch_bounds__(LeafShape<NW>::threads, LeafShape<NW>::min_blo
 
 size_t tree_node_words() { return (size_t)kNW; }
 
-cudaError_t launch_tree_bound(const uint32_t* ms, const uint8_t* fe, uint32_t n, uint32_t* bound, TreeCounters* ctr,
+cudaError_t launch_tree_bound(const uint32_t* ms, const uint8_t* fe, uint32_t n, TreeBounds* bounds, TreeCounters* ctr,
                               cudaStream_t st) {
-  tree_bound_kernel<<<1, 1, 0, st>>>(ms, fe, n, bound, ctr);
+  tree_bound_kernel<<<1, 1, 0, st>>>(ms, fe, n, bounds, ctr);
   return cudaGetLastError();
 }
 
 cudaError_t launch_tree_start(const TablesW& tb, const TreeConsts& tc, uint32_t d0, TreeLevel dst, uint32_t cap,
-                              const uint32_t* bound, TreeCounters* ctr, cudaStream_t st) {
+                              TreeBounds* bounds, TreeCounters* ctr, cudaStream_t st) {
   uint32_t combos = 1;
   for (uint32_t i = 0; i < d0; ++i) combos *= tc.radix;
   tree_start_kernel<<<(combos + kTreeThreads - 1) / kTreeThreads, kTreeThreads, 0, st>>>(tb, tc, d0, combos, dst, cap,
-                                                                                         bound, ctr);
+                                                                                         bounds, ctr);
   return cudaGetLastError();
 }
 
 cudaError_t launch_tree_expand(const TablesW& tb, const TreeConsts& tc, TreeLevel src, uint32_t pop,
-                               uint32_t most_nodes, uint32_t d, TreeLevel dst, uint32_t cap, const uint32_t* bound,
+                               uint32_t most_nodes, uint32_t d, TreeLevel dst, uint32_t cap, TreeBounds* bounds,
                                TreeCounters* ctr, cudaStream_t st) {
   const uint64_t threads = (uint64_t)(most_nodes < pop ? most_nodes : pop) * tc.radix;
   const unsigned grid = (unsigned)((threads + kTreeThreads - 1) / kTreeThreads);
-  tree_expand_kernel<<<grid, kTreeThreads, 0, st>>>(tb, tc, src, pop, d, dst, cap, bound, ctr);
+  tree_expand_kernel<<<grid, kTreeThreads, 0, st>>>(tb, tc, src, pop, d, dst, cap, bounds, ctr);
   return cudaGetLastError();
 }
 
 template <int NW>
 static cudaError_t leaf_launch(const TablesW& tb, const TreeConsts& tc, TreeLevel src, uint32_t cap,
-                               uint32_t most_nodes, uint32_t* bound, BestRecord* best, TreeCounters* ctr,
+                               uint32_t most_nodes, TreeBounds* bounds, BestRecord* best, TreeCounters* ctr,
                                cudaStream_t st) {
   static std::atomic<uint64_t> ready{0};
   const size_t smem = sizeof(uint32_t) * LaneWords<NW>::value * LeafShape<NW>::threads;
@@ -265,16 +272,16 @@ static cudaError_t leaf_launch(const TablesW& tb, const TreeConsts& tc, TreeLeve
   const uint64_t need = (tasks + LeafShape<NW>::warps - 1) / LeafShape<NW>::warps;
   const uint64_t most = (uint64_t)sms * LeafShape<NW>::min_blocks * 8u;
   tree_leaf_kernel<NW><<<(unsigned)(need < most ? need : most), LeafShape<NW>::threads, smem, st>>>(
-      tb, tw, tc, src, cap, bound, best, ctr);
+      tb, tw, tc, src, cap, bounds, best, ctr);
   return cudaGetLastError();
 }
 
 cudaError_t launch_tree_leaf(const TablesW& tb, const TreeConsts& tc, TreeLevel src, uint32_t cap,
-                             uint32_t most_nodes, uint32_t* bound, BestRecord* best, TreeCounters* ctr,
+                             uint32_t most_nodes, TreeBounds* bounds, BestRecord* best, TreeCounters* ctr,
                              cudaStream_t st) {
   const uint32_t nw = tb.n - tc.W0;
 #define BF_TRY(NW) \
-  if (nw <= (uint32_t)NW) return leaf_launch<NW>(tb, tc, src, cap, most_nodes, bound, best, ctr, st);
+  if (nw <= (uint32_t)NW) return leaf_launch<NW>(tb, tc, src, cap, most_nodes, bounds, best, ctr, st);
   BF_TREE_BUCKETS(BF_TRY)
 #undef BF_TRY
   return cudaErrorInvalidValue;

@@ -481,6 +481,16 @@ __device__ __forceinline__ Digits leaf_mode_digits(const LeafModes& modes, const
   return d;
 }
 
+// The makespans a search prunes by, in device memory.  `live` is the best one
+// known; the blocks of a leaf launch lower it while others of the same launch
+// start.  `leaf` is what `live` was before the coming leaf launch (the start and
+// expansion kernels copy it, and only leaf launches change `live`): the tasks
+// of a node group cut one list of combinations into parts, so that list must be
+// the same for all of them.
+struct TreeBounds {
+  uint32_t live, leaf;
+};
+
 __device__ __forceinline__ uint32_t read_bound(const uint32_t* bound) {
   return *reinterpret_cast<const volatile uint32_t*>(bound);
 }
@@ -498,6 +508,9 @@ __device__ __forceinline__ uint32_t read_bound(const uint32_t* bound) {
 // / dealt only / by this rule: 14 layered tools 0.87 / 0.77 / 0.60 ms, 18 tools
 // 1.28 / 1.36 / 1.05, 26 tools 2.13 / 1.92 / 1.80; binary space of 24 tools 1.20 /
 // 5.5 / 1.00 (dealt lanes leave the common path).
+// Modes, totals and that choice depend on the nodes and on bounds->leaf alone, so
+// that the parts of a group are parts of one list whenever they run; the live
+// bound only gives up single runs.
 // `slot`: this lane's window state in shared memory (stride STRIDE, the warp's 32
 // lanes side by side).  Every lane of the warp calls it.  Returns the
 // combinations this lane simulated; *nodes has the lanes with a node to enumerate.
@@ -505,19 +518,21 @@ template <int NW, uint32_t STRIDE, typename TB, typename TBW, typename SD>
 __device__ __forceinline__ uint32_t leaf_task(const TB& tb, const TBW& tw, const SD& sdw, const uint32_t* rtw,
                                               const TreeConsts& tc, const uint32_t* buf, uint32_t cap, uint32_t cnt,
                                               uint32_t g, uint32_t part, uint32_t parts, uint32_t chunk,
-                                              const uint32_t* bound, uint32_t* slot, LaneBest& best, uint32_t* nodes) {
+                                              const TreeBounds* bounds, uint32_t* slot, LaneBest& best,
+                                              uint32_t* nodes) {
   const uint32_t lane = threadIdx.x & 31u, j = g * 32u + lane;
   bool valid = j < cnt;
   Digits dg{0u, 0u};
   LeafModes modes{0u, 0u, 0u};
-  uint32_t limit = tc.prune ? read_bound(bound) : kInfeasible;
+  const uint32_t kept = tc.prune ? read_bound(&bounds->leaf) : kInfeasible;
+  uint32_t limit = kept;  // of single runs: falls with the live bound
   __syncwarp();  // the other lanes are done with this lane's state
   if (valid) {
     const uint32_t* t = buf + j + (size_t)(2 * kTreeSlots) * cap;
     dg = Digits{t[9 * (size_t)cap], t[10 * (size_t)cap]};
     // The incumbent may have improved since this node was bounded; only modes
     // within it are enumerated.
-    if (tc.prune) valid = node_leaf_modes(buf, cap, j, tb, tc, dg, limit, slot, STRIDE, &modes);
+    if (tc.prune) valid = node_leaf_modes(buf, cap, j, tb, tc, dg, kept, slot, STRIDE, &modes);
     if (valid) node_to_window<NW>(buf, cap, j, tc.W0, tw.n, slot, STRIDE);
   }
   __syncwarp();  // dealt combinations resume other lanes' states: votes and shuffles order no memory
@@ -545,7 +560,7 @@ __device__ __forceinline__ uint32_t leaf_task(const TB& tb, const TBW& tw, const
                         __shfl_sync(0xFFFFFFFFu, modes.que, i)};
       const Digits d{__shfl_sync(0xFFFFFFFFu, dg.now, i), __shfl_sync(0xFFFFFFFFu, dg.que, i)};
       if (base + lane < q1) {
-        limit = min(limit, read_bound(bound));
+        limit = min(limit, read_bound(&bounds->live));
         const Digits dc = leaf_mode_digits(m, tc, q - (i ? before : 0u));
         ran += leaf_run<NW>(tw, sdw, rtw, tc, slot + (int)(i - lane), STRIDE, d, dc, best, limit) ? 1u : 0u;
       }
@@ -556,7 +571,7 @@ __device__ __forceinline__ uint32_t leaf_task(const TB& tb, const TBW& tw, const
     const uint32_t rounds = __reduce_max_sync(0xFFFFFFFFu, q1 - q0);
     for (uint32_t k = 0; k < rounds; ++k) {
       if (q0 + k < q1) {
-        limit = min(limit, read_bound(bound));
+        limit = min(limit, read_bound(&bounds->live));
         ran += leaf_run<NW>(tw, sdw, rtw, tc, slot, STRIDE, dg, leaf_mode_digits(modes, tc, q0 + k), best, limit) ? 1u : 0u;
       }
       __syncwarp();

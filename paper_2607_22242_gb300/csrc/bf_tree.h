@@ -35,21 +35,22 @@ struct TreeLevel {
 
 size_t tree_node_words();
 // The starting bound: the least feasible of n candidates' makespans
-// (0xFFFFFFFF without one), to *bound and ctr->incumbent.
-cudaError_t launch_tree_bound(const uint32_t* ms, const uint8_t* fe, uint32_t n, uint32_t* bound, TreeCounters* ctr,
+// (0xFFFFFFFF without one), to bounds->live and ctr->incumbent.
+cudaError_t launch_tree_bound(const uint32_t* ms, const uint8_t* fe, uint32_t n, TreeBounds* bounds, TreeCounters* ctr,
                               cudaStream_t st);
 // Append the surviving nodes of the first d0 tools' modes to `dst` (level d0).
 cudaError_t launch_tree_start(const TablesW& tb, const TreeConsts& tc, uint32_t d0, TreeLevel dst, uint32_t cap,
-                              const uint32_t* bound, TreeCounters* ctr, cudaStream_t st);
+                              TreeBounds* bounds, TreeCounters* ctr, cudaStream_t st);
 // Expand the last min(*src.count, pop) nodes of `src` (level d, at most
 // most_nodes of them) into `dst`; the counts are read on the device, so that
 // launches follow one another without the host.
 cudaError_t launch_tree_expand(const TablesW& tb, const TreeConsts& tc, TreeLevel src, uint32_t pop,
-                               uint32_t most_nodes, uint32_t d, TreeLevel dst, uint32_t cap, const uint32_t* bound,
+                               uint32_t most_nodes, uint32_t d, TreeLevel dst, uint32_t cap, TreeBounds* bounds,
                                TreeCounters* ctr, cudaStream_t st);
-// Enumerate the leaves of every node of `src`, the leaf level.
+// Enumerate the leaves of every node of `src`, the leaf level.  A start or an
+// expansion must have run since the last launch of this (TreeBounds::leaf).
 cudaError_t launch_tree_leaf(const TablesW& tb, const TreeConsts& tc, TreeLevel src, uint32_t cap,
-                             uint32_t most_nodes, uint32_t* bound, BestRecord* best, TreeCounters* ctr,
+                             uint32_t most_nodes, TreeBounds* bounds, BestRecord* best, TreeCounters* ctr,
                              cudaStream_t st);
 
 }  // namespace bfk

@@ -113,7 +113,7 @@ struct LeafLevel {
 };
 
 template <int NW>
-int leaf_warps(const LeafLevel& L, uint32_t parts, const uint32_t* bounds, uint64_t* out) {
+int leaf_warps(const LeafLevel& L, uint32_t start, uint32_t parts, const uint32_t* bounds, uint64_t* out) {
   const TreeConsts& tc = L.tc;
   TablesT<NW> tw;
   host::build_window(L.tb, tc.W0, &tw);
@@ -126,7 +126,7 @@ int leaf_warps(const LeafLevel& L, uint32_t parts, const uint32_t* bounds, uint6
   uint64_t ms = ~0ull, idx = ~0ull, ran = 0, nodes = 0;
   for (uint32_t g = 0; g < (L.count + 31u) / 32u; ++g)
     for (uint32_t part = 0; part < parts; ++part) {
-      uint32_t bound = bounds[part];
+      const TreeBounds bound{bounds[part], start};
       const int err = hostwarp::run(stale, [&](unsigned lane) {
         LaneBest best;
         uint32_t live;
@@ -154,8 +154,8 @@ int leaf_warps(const LeafLevel& L, uint32_t parts, const uint32_t* bounds, uint6
 }  // namespace
 
 // The leaf kernel's tasks over every leaf node that the expansions keep from
-// `start`, `parts` tasks per group of 32 nodes, task p under the bound
-// bounds[p].  out[0..4] = best makespan (~0: none), its canonical index,
+// `start`, which is also the leaf launch's bound, `parts` tasks per group of 32
+// nodes, task p with the live bound at bounds[p].  out[0..4] = best makespan (~0: none), its canonical index,
 // mappings simulated, nodes enumerated by the groups' first tasks, leaf nodes.
 extern "C" int host_leaf_warps(const bf_scenario_desc* d, uint32_t space, int prune, uint32_t start, uint32_t parts,
                                const uint32_t* bounds, uint64_t* out) {
@@ -164,7 +164,7 @@ extern "C" int host_leaf_warps(const bf_scenario_desc* d, uint32_t space, int pr
   const LeafLevel L(d, space, prune != 0, start);
   const uint32_t nw = L.tb.n - L.tc.W0;
 #define BF_TRY(NW) \
-  if (nw <= (uint32_t)NW) return leaf_warps<NW>(L, parts, bounds, out);
+  if (nw <= (uint32_t)NW) return leaf_warps<NW>(L, start, parts, bounds, out);
   BF_TREE_BUCKETS(BF_TRY)
 #undef BF_TRY
   return -1;

@@ -74,3 +74,28 @@ def test_leaf_tasks_share_nodes(warp, n, parts):
                 assert got[0] == want, (t, space, start, got, want)
             if n <= 8:
                 assert _leaves(warp, scn, space, 0xFFFFFFFF, [0xFFFFFFFF] * parts, prune=False)[0] == want
+
+
+def _layered(n, seed):
+    """A layered DAG (layers of 4, edge probability 0.4) with the standard profile recipe, 24 GiB."""
+    rng = np.random.default_rng(seed)
+    c, g, x, m = S._ordinary(np.random.default_rng([seed, n]), n, 2048, 16384)
+    pred = S._layered_edges(rng, [4] * (n // 4) + ([n % 4] if n % 4 else []), 0.4)
+    return S.Scenario(n, pred, c, g, x, [S._load_from_vram(v) for v in m], m, 24576, S.slowdown_linear(kmax=n))
+
+
+@pytest.mark.parametrize("n,seed", [(11, 0), (12, 1), (13, 3)])
+@pytest.mark.parametrize("parts", [2, 5, 16])
+def test_leaf_tasks_while_the_bound_improves(warp, n, seed, parts):
+    """The best makespan improves between the tasks of a node group, at every place among them (from 5 % above the
+    optimum to the optimum): the optimum is found all the same, and the tasks simulate as many combinations in all as
+    without the improvement -- the parts stay those of one list."""
+    scn = _layered(n, seed)
+    opt = oracle.search(scn, THREADS)
+    loose = opt[1] + opt[1] // 20
+    want = _leaves(warp, scn, 3, loose, [loose] * parts)
+    assert want[0] == opt
+    for k in range(parts + 1):
+        got = _leaves(warp, scn, 3, loose, [loose] * k + [opt[1]] * (parts - k))
+        assert got[0] == opt, k
+        assert got[1:] == want[1:], k
