@@ -404,8 +404,9 @@ struct LaneBest {
 // Simulate one combination `dc` of the leaf tools' modes (bit 0: tool L) of the
 // leaf node saved in `slot` (a lane's shared-memory window state, stride
 // `stride`) whose digits are `dg` (all tools); tw/sdw/rtw are the window's
-// tables.  A run past `bound` or the best so far is given up; false when the
-// combination was not simulated (a queued tool larger than the budget).
+// tables.  A run past `bound` is given up, and when pruning one past the best so
+// far; false when the combination was not simulated (a queued tool larger than
+// the budget).
 // With tc.alone_last, dc are modes of the leaf tools but the last one: the run
 // goes on until the last tool becomes ready (everything else has ended then)
 // and yields one makespan per mode of the last tool.
@@ -419,7 +420,7 @@ __device__ __forceinline__ bool leaf_run(const TBW& tw, const SD& sdw, const uin
   if (sim.que & tw.big_mask) return false;
   State<NW> w;
   load_lane(slot, stride, w);
-  const uint32_t limit = best.ms < bound ? best.ms : bound;
+  const uint32_t limit = tc.prune && best.ms < bound ? best.ms : bound;
   if (tc.alone_last) {
     if (run<NW>(w, tw, sdw, rtw, sim, 1u << lastw, 1u << lastw, limit) != kRunStopped) return true;  // infeasible before it
     for (uint32_t a = 0; a < tc.radix; ++a) {

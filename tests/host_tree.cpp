@@ -140,3 +140,64 @@ extern "C" int host_tree(const bf_scenario_desc* d, uint32_t space, uint32_t pru
 #undef BF_TRY
   return -1;
 }
+
+// How many steps with a GPU tool running the unpruned leaf enumeration takes
+// (leaf_combos), over every leaf node: with one LaneBest for all of a node's
+// combinations as a lane has it, or (`fresh`) with a new one for each.
+namespace {
+struct Counted {  // reads of the slowdown table, one per such step
+  const uint32_t* p;
+  uint64_t* reads;
+  uint32_t operator[](uint32_t k) const { ++*reads; return p[k]; }
+};
+template <int NW>
+struct CountedTables {
+  Counted f;
+  const uint64_t* recip;
+  const uint32_t* pred;
+};
+
+template <int NW>
+struct Steps {
+  const TablesW& tb;
+  const TreeConsts& tc;
+  Search<NW>& t;
+  bool fresh;
+  uint64_t reads = 0;
+
+  void visit(const State<kTreeSlots>& s, Digits dg, uint32_t d) {
+    if (d == tc.leaf_level) {
+      store_node(s, dg, t.node.data(), 1u, 0u);
+      node_to_window<NW>(t.node.data(), 1u, 0u, tc.W0, t.tw.n, t.slot.data(), 1u);
+      const CountedTables<NW> sd{{t.sdw.f, &reads}, t.sdw.recip, t.sdw.pred};
+      const uint32_t ncomb = tc.alone_last ? tc.combos / tc.radix : tc.combos;
+      LaneBest lb;
+      for (uint32_t c = 0; c < ncomb; ++c) {
+        if (fresh) lb = LaneBest{};
+        leaf_combos<NW>(t.tw, sd, t.rtw.data(), tc, t.slot.data(), 1u, dg, true, c, c + 1u, lb);
+      }
+      return;
+    }
+    for (uint32_t a = 0; a < tc.radix; ++a) {
+      State<kTreeSlots> c = s;
+      Digits cd = dg;
+      if (expand_child<kTreeSlots>(tb, t.sd, t.rt.data(), tc, c, cd, d, a, kInfeasible, t.ef.data(), 1u))
+        visit(c, cd, d + 1);
+    }
+  }
+};
+}  // namespace
+
+extern "C" uint64_t host_unpruned_steps(const bf_scenario_desc* d, uint32_t space, int fresh) {
+  TablesW t0, tb;
+  host::build_tables(d, &t0);
+  host::relabel_sources_first(t0, &tb);
+  TreeConsts tc;
+  host::tree_consts(tb, space, false, &tc);
+  Search<32> search(tb, tc, kInfeasible);
+  Steps<32> steps{tb, tc, search, fresh != 0};
+  State<kTreeSlots> s;
+  init_state(s, tb.all_mask);
+  steps.visit(s, Digits{0u, 0u}, 0u);
+  return steps.reads;
+}

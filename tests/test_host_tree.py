@@ -44,6 +44,9 @@ def tree():
         ms, idx = int(res[0]), int(res[1])
         best = (idx, ms) if ms != 2 ** 64 - 1 else (-1, INF)
         return best, res[2:].tolist()
+    lib.host_unpruned_steps.argtypes = [ctypes.POINTER(bf.Desc), ctypes.c_uint32, ctypes.c_int]
+    lib.host_unpruned_steps.restype = ctypes.c_uint64
+    run.unpruned_steps = lambda scn, space, fresh: lib.host_unpruned_steps(ctypes.byref(bf.to_desc(scn)), space, fresh)
     return run
 
 
@@ -166,3 +169,18 @@ def test_tree_node_logic_beyond_20_tools(tree):
         if name == "layered24":
             assert st[2] == 1
     assert max(widths) > 12, widths  # a leaf window wider than the small DAGs reach
+
+
+@pytest.mark.parametrize("n", [5, 8])
+@pytest.mark.parametrize("joined", [False, True])
+def test_unpruned_search_simulates_every_mapping_to_its_end(tree, n, joined):
+    """Without pruning no run is given up at the best makespan so far: a lane's enumeration takes the steps of
+    simulations that know nothing of one another."""
+    rng = np.random.default_rng(n)
+    for t in range(4):
+        scn = S.random_small(rng, n, edge_p=0.2, tight=bool(t % 2), contention=True, max_time=40)
+        if joined:
+            scn = _with_last_waiting(scn, n)
+        for space in (3, 2):
+            steps = tree.unpruned_steps(scn, space, 1)
+            assert tree.unpruned_steps(scn, space, 0) == steps > 0, (t, space)
