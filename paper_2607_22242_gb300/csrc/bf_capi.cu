@@ -131,59 +131,13 @@ int current_ctx_id(unsigned long long* id, const char* who) {
   return BF_OK;
 }
 
-// Scratch of handles that are gone (a device block and its pinned mirror, 14 KB
-// each), for the next handles: allocating and freeing them took most of a
-// one-off search (12-tool fan-out through bf_create_scenario, bf_search_best
-// and bf_destroy_scenario: 547 -> 118 us).  At most kMost pairs are kept; a pair
-// belongs to the context it was made in and is only handed out there.
-class ScratchPool {
- public:
-  struct Pair {
-    bf_scratch* d;
-    bf_scratch* h;
-  };
-
-  // A pair made in the current context, or false.
-  bool take(Pair* out) {
-    unsigned long long id = 0;
-    if (!context(&id)) return false;
-    std::lock_guard<std::mutex> lock(mu_);
-    for (unsigned i = 0; i < count_; ++i)
-      if (slots_[i].ctx == id) {
-        *out = slots_[i].pair;
-        slots_[i] = slots_[--count_];
-        return true;
-      }
-    return false;
-  }
-
-  // Keep a pair of the current context; false (the caller frees it) when the
-  // pool is full or the context cannot be told.
-  bool keep(const Pair& pair) {
-    unsigned long long id = 0;
-    if (!context(&id)) return false;
-    std::lock_guard<std::mutex> lock(mu_);
-    if (count_ == kMost) return false;
-    slots_[count_++] = Slot{id, pair};
-    return true;
-  }
-
- private:
-  static constexpr unsigned kMost = 16;
-  struct Slot {
-    unsigned long long ctx;
-    Pair pair;
-  };
-  static bool context(unsigned long long* id) {
-    const CtxFns& f = ctx_fns();
-    CUcontext ctx = nullptr;
-    return f.get_current && f.get_id && f.get_current(&ctx) == CUDA_SUCCESS && ctx && f.get_id(ctx, id) == CUDA_SUCCESS;
-  }
-  std::mutex mu_;
-  Slot slots_[kMost];
-  unsigned count_ = 0;
-};
-ScratchPool g_scratch_pool;
+// ID of the current context; false when there is none or it cannot be told.
+bool scratch_context(unsigned long long* id) {
+  const CtxFns& f = ctx_fns();
+  CUcontext ctx = nullptr;
+  return f.get_current && f.get_id && f.get_current(&ctx) == CUDA_SUCCESS && ctx && f.get_id(ctx, id) == CUDA_SUCCESS;
+}
+ScratchPool<bf_scratch> g_scratch_pool(scratch_context);
 
 int validate(const bf_scenario_desc* d, const char* who) {
   if (!d) return fail(BF_EINVAL, "%s: desc is NULL", who);
@@ -233,11 +187,11 @@ int wait_stream(cudaStream_t st, const char* who) {
   }
 }
 
-void begin_call(const bf_scenario* scn) { const_cast<bf_scenario*>(scn)->busy = true; }
+void begin_call(const bf_scenario* scn) { const_cast<bf_scenario*>(scn)->calls.begin(); }
 
 int end_call(const bf_scenario* scn, cudaStream_t st, const char* who) {
   const int rc = wait_stream(st, who);
-  if (rc == BF_OK) const_cast<bf_scenario*>(scn)->busy = false;
+  if (rc == BF_OK) const_cast<bf_scenario*>(scn)->calls.end();
   return rc;
 }
 
@@ -593,7 +547,7 @@ int bf_create_scenario(const bf_scenario_desc* desc, bf_scenario** out) {
       s->lt_x = ltrec.x;
     }
   }
-  ScratchPool::Pair pair{nullptr, nullptr};
+  ScratchPool<bf_scratch>::Pair pair{nullptr, nullptr};
   if (e == cudaSuccess && !g_scratch_pool.take(&pair)) {
     e = lib_malloc(reinterpret_cast<void**>(&pair.d), sizeof(bf_scratch));
     if (e == cudaSuccess) e = lib_malloc_host(reinterpret_cast<void**>(&pair.h), sizeof(bf_scratch));
@@ -639,7 +593,7 @@ int bf_destroy_scenario(bf_scenario* scn) {
   // cudaFree waits for it.
   int device = -1;
   const bool here = cudaGetDevice(&device) == cudaSuccess && device == scn->device;
-  if (!here || scn->busy || !g_scratch_pool.keep({scn->d_scratch, scn->h_scratch})) {
+  if (!here || !scn->calls.none_open() || !g_scratch_pool.keep({scn->d_scratch, scn->h_scratch})) {
     const cudaError_t e = cudaFree(scn->d_scratch);
     if (e1 == cudaSuccess) e1 = e;
     e2 = cudaFreeHost(scn->h_scratch);
@@ -858,7 +812,7 @@ int bf_search_pruned(const bf_scenario* scn_const, uint64_t hint_index, bf_resul
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(&h->survivors, &dv->survivors, 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, st);
   if (e != cudaSuccess) return cuda_fail(e, who);
-  int rc = wait_stream(st, who);
+  int rc = end_call(scn, st, who);
   if (rc != BF_OK) return rc;
   plan.bound = h->pruned_bound;
   const uint32_t nsurv = h->survivors;
@@ -871,6 +825,7 @@ int bf_search_pruned(const bf_scenario* scn_const, uint64_t hint_index, bf_resul
   //    inner checkpoint; tasks of at least 16 mid combinations, about
   //    kSearchTasks of them.
   plan.groups = (nsurv + 31u) / 32u;
+  begin_call(scn);
   e = cudaMemsetAsync(scn->d_key, 0xFF, sizeof(unsigned long long), st);
   if (e == cudaSuccess && nsurv) {
     const uint64_t num_m = (uint64_t)plan.m_hi - plan.m_lo + 1;

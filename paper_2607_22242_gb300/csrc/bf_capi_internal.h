@@ -11,6 +11,7 @@
 #include "bf_lanetree_launch.h"
 #include "bf_launch.h"
 #include "bf_plan.h"
+#include "bf_scratch_pool.h"
 #include "bf_segments.h"
 #include "bf_tree.h"
 
@@ -68,7 +69,7 @@ struct bf_scenario {
   uint32_t* d_survivors;      // pruned search: 3^pplan.P prefix slots, allocated on first use
   uint32_t* d_levels;         // tree search: node buffers of every level, allocated on first use
   size_t levels_bytes;
-  bool busy;                  // a call's work may be in flight (also after one that failed or timed out)
+  bfcapi::OpenCalls calls;    // whose work may be in flight (also after one that failed or timed out)
 };
 
 namespace bfcapi {

@@ -1,4 +1,8 @@
-"""Handles made and destroyed one after the other, and by several threads at once, share pooled scratch (GPU)."""
+"""Handles made and destroyed one after the other, and by several threads at once, share pooled scratch (GPU); the
+pool's own rules without one."""
+import ctypes
+import os
+import subprocess
 import threading
 
 import pytest
@@ -65,3 +69,49 @@ def test_a_handle_closed_after_a_timeout_keeps_its_scratch_to_itself():
     finally:
         bf.set_wait_timeout_ms(600000)
         torch.cuda.synchronize()
+
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def pool(tmp_path_factory):
+    out = str(tmp_path_factory.mktemp("pool") / "host_pool.so")
+    subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-o", out, os.path.join(HERE, "host_pool.cpp")],
+                   check=True)
+    return ctypes.CDLL(out)
+
+
+@pytest.mark.parametrize("calls,may", [(b"", 1), (b"be", 1), (b"bebe", 1), (b"b", 0),
+                                       (b"bbe", 0),      # a good call after one that stopped waiting
+                                       (b"bebbebe", 0)])
+def test_scratch_of_an_unfinished_call_is_never_kept(pool, calls, may):
+    assert pool.host_may_keep(calls) == may
+
+
+@pytest.mark.gpu
+def test_a_good_call_after_a_timeout_does_not_release_the_scratch():
+    """A search whose wait ran out, then a good call on another stream beside it: closing the handle waits for the
+    search instead of handing its scratch on, and the next handles' results are right."""
+    import torch
+    scn, small = S.config3(), S.config0()
+    slow, fast = torch.cuda.Stream(), torch.cuda.Stream(priority=-1)
+    beside = 0
+    try:
+        for _ in range(5):
+            h = bf.create_scenario(scn)
+            bf.set_wait_timeout_ms(1)
+            with pytest.raises(bf.BfError) as ei:
+                bf.search_best(h, slow)
+            assert ei.value.code == bf.BF_ETIMEOUT
+            bf.set_wait_timeout_ms(600000)
+            bf.whatif(h, 0, stream=fast)
+            beside += not slow.query()  # the search was still running when the good call ended
+            h.close()
+            assert slow.query()
+            r = bf.search_best(small)
+            assert (r.index, r.makespan_us) == oracle.search(small)
+    finally:
+        bf.set_wait_timeout_ms(600000)
+        torch.cuda.synchronize()
+    assert beside > 0
