@@ -554,6 +554,7 @@ int bf_create_scenario(const bf_scenario_desc* desc, bf_scenario** out) {
   }
   s->d_scratch = pair.d;
   s->h_scratch = pair.h;
+  s->ctx = g_scratch_pool.context();
   if (e != cudaSuccess) {
     const int code = cuda_fail(e, "bf_create_scenario");
     if (s->d_scratch) cudaFree(s->d_scratch);
@@ -593,7 +594,7 @@ int bf_destroy_scenario(bf_scenario* scn) {
   // cudaFree waits for it.
   int device = -1;
   const bool here = cudaGetDevice(&device) == cudaSuccess && device == scn->device;
-  if (!here || !scn->calls.none_open() || !g_scratch_pool.keep({scn->d_scratch, scn->h_scratch})) {
+  if (!here || !scn->calls.none_open() || !g_scratch_pool.keep({scn->d_scratch, scn->h_scratch}, scn->ctx)) {
     const cudaError_t e = cudaFree(scn->d_scratch);
     if (e1 == cudaSuccess) e1 = e;
     e2 = cudaFreeHost(scn->h_scratch);

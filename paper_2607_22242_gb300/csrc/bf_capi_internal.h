@@ -61,6 +61,7 @@ struct bf_scenario {
   bfk::SegPlan seg;
   uint32_t* d_table;
   int device;
+  unsigned long long ctx;     // ID of the context the scratch was made in, 0 when it could not be told
   bf_scratch* d_scratch;      // device scratch
   bf_scratch* h_scratch;      // pinned host mirror
   unsigned long long* d_key;  // &d_scratch->key

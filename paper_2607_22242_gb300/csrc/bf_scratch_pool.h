@@ -23,7 +23,7 @@ struct OpenCalls {
 // took most of a one-off search (12-tool fan-out through bf_create_scenario,
 // bf_search_best and bf_destroy_scenario: 547 -> 118 us).  At most kMost pairs
 // are kept; a pair belongs to the context it was made in and is only handed out
-// there.  `context` gives the ID of the current context, or false.
+// there.  `context` gives the ID of the current context (never 0), or false.
 template <typename Scratch>
 class ScratchPool {
  public:
@@ -35,10 +35,16 @@ class ScratchPool {
 
   explicit ScratchPool(ContextFn context) : context_(context) {}
 
+  // ID of the current context, 0 when it cannot be told.
+  unsigned long long context() const {
+    unsigned long long id = 0;
+    return context_(&id) ? id : 0;
+  }
+
   // A pair made in the current context, or false.
   bool take(Pair* out) {
-    unsigned long long id = 0;
-    if (!context_(&id)) return false;
+    const unsigned long long id = context();
+    if (id == 0) return false;
     std::lock_guard<std::mutex> lock(mu_);
     for (unsigned i = 0; i < count_; ++i)
       if (slots_[i].ctx == id) {
@@ -49,14 +55,14 @@ class ScratchPool {
     return false;
   }
 
-  // Keep a pair of the current context; false (the caller frees it) when the
-  // pool is full or the context cannot be told.
-  bool keep(const Pair& pair) {
-    unsigned long long id = 0;
-    if (!context_(&id)) return false;
+  // Keep a pair made in context `made_in`; false (the caller frees it) when the
+  // pool is full or another context is current: the device may have been reset
+  // since, and the pair be gone.
+  bool keep(const Pair& pair, unsigned long long made_in) {
+    if (made_in == 0 || made_in != context()) return false;
     std::lock_guard<std::mutex> lock(mu_);
     if (count_ == kMost) return false;
-    slots_[count_++] = Slot{id, pair};
+    slots_[count_++] = Slot{made_in, pair};
     return true;
   }
 

@@ -89,6 +89,20 @@ def test_scratch_of_an_unfinished_call_is_never_kept(pool, calls, may):
     assert pool.host_may_keep(calls) == may
 
 
+def test_pairs_stay_in_the_context_they_were_made_in(pool):
+    """A pair is handed out only where it was made, also when its handle is destroyed under another context (after a
+    device reset, say): such a pair is not kept at all, nor one whose context could not be told."""
+    pool.host_keep.argtypes = [ctypes.c_void_p, ctypes.c_uint64, ctypes.c_uint64]
+    pool.host_take.argtypes, pool.host_take.restype = [ctypes.c_uint64], ctypes.c_void_p
+    assert pool.host_keep(16, 1, 1) == 1
+    assert pool.host_keep(32, 1, 2) == 0
+    assert pool.host_keep(48, 0, 2) == 0 and pool.host_keep(48, 0, 0) == 0
+    assert pool.host_take(2) is None and pool.host_take(0) is None
+    assert pool.host_take(1) == 16 and pool.host_take(1) is None
+    kept = [pool.host_keep(16 * k, 3, 3) for k in range(1, 40)]
+    assert sum(kept) == 16  # bounded
+
+
 @pytest.mark.gpu
 def test_a_good_call_after_a_timeout_does_not_release_the_scratch():
     """A search whose wait ran out, then a good call on another stream beside it: closing the handle waits for the
