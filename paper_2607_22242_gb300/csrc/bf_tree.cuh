@@ -112,81 +112,13 @@ __device__ __forceinline__ void load_node(const uint32_t* buf, uint32_t cap, uin
   dg.que = p[10 * (size_t)cap];
 }
 
-// Lower bound on the makespan of every mapping that extends a node whose
-// state `s` is at a checkpoint (before the admission at s.T), with the modes
-// of the tools in `known` given by `dg`:
-//   * a running CPU tool ends at ec (exact);
-//   * a running GPU tool with r work units left ends no earlier than
-//     T + ceil(r / 1024): f[k] >= f[1] = 1024, and the model rounds GPU
-//     progress down and completion times up;
-//   * a tool not started by T ends no earlier than T + its duration in its
-//     mode (c, g + x or l + g + x), or T + min(c, g + x) if its mode is open;
-//   * after a tool ends, its successors still need the longest path through
-//     them in minimum durations (sdown);
-//   * queued tools run one at a time, so all unfinished tools known to be
-//     queued end no earlier than T + the sum of their remaining durations.
-template <int NT, typename TB, typename Slots>
-__device__ __forceinline__ uint64_t lower_bound_of(uint32_t done, uint32_t run_g, uint32_t T32, uint32_t V,
-                                                   const Slots& slot, const TB& tb, const TreeConsts& tc, Digits dg,
-                                                   uint32_t known) {
-  const uint64_t T = T32;
-  uint64_t lb = T, qsum = 0u;
-#pragma unroll
-  for (int v = 0; v < NT; ++v) {
-    const uint32_t bit = 1u << v;
-    if (done & bit) continue;
-    const uint32_t ec = slot.ec(v);
-    uint64_t fin;
-    if (ec != 0xFFFFFFFFu) {
-      fin = ec;
-    } else if (run_g & bit) {
-      const uint32_t r = slot.eg(v) - V;
-      const uint32_t left = (r >> 10) + ((r & 1023u) != 0u);
-      fin = T + left;
-      if (dg.que & bit) qsum += left;
-    } else {
-      uint32_t d = tc.dmin[v];
-      if (known & bit) {
-        d = (dg.now & bit) ? (tb.wnow[v] >> 10) : (dg.que & bit) ? (tb.wq[v] >> 10) : tb.cpu[v];
-        if (dg.que & bit) qsum += d;
-      }
-      fin = T + d;
-    }
-    lb = max(lb, fin + tc.sdown[v]);
-  }
-  return max(lb, T + qsum);
-}
-
-// Per-slot end times of a state held in registers, or of a node saved in HBM.
-template <int NT>
-struct StateSlots {
-  const State<NT>& s;
-  __device__ __forceinline__ uint32_t ec(int v) const { return s.ec[v]; }
-  __device__ __forceinline__ uint32_t eg(int v) const { return s.eg[v]; }
-};
-
+// Per-slot end times of a node saved in HBM.
 struct NodeSlots {
   const uint32_t* p;  // word 0 of the node
   uint32_t cap;
   __device__ __forceinline__ uint32_t ec(int v) const { return p[(size_t)(2 * v) * cap]; }
   __device__ __forceinline__ uint32_t eg(int v) const { return p[(size_t)(2 * v + 1) * cap]; }
 };
-
-template <int NT, typename TB>
-__device__ __forceinline__ uint64_t lower_bound(const State<NT>& s, const TB& tb, const TreeConsts& tc, Digits dg,
-                                                uint32_t known) {
-  return lower_bound_of<NT>(s.done, s.run_g, s.T, s.V, StateSlots<NT>{s}, tb, tc, dg, known);
-}
-
-// The bound of node j of a level buffer, read word by word from HBM.
-template <typename TB>
-__device__ __forceinline__ uint64_t node_lower_bound(const uint32_t* buf, uint32_t cap, uint32_t j, const TB& tb,
-                                                     const TreeConsts& tc, Digits dg, uint32_t known) {
-  const uint32_t* p = buf + j;
-  const uint32_t* t = p + (size_t)(2 * kTreeSlots) * cap;
-  return lower_bound_of<kTreeSlots>(t[0], t[2 * (size_t)cap], t[4 * (size_t)cap], t[5 * (size_t)cap],
-                                    NodeSlots{p, cap}, tb, tc, dg, known);
-}
 
 // Copy node j of a level buffer into a lane's shared-memory state over the
 // window [W0, W0 + NW) (slots past the last tool: no CPU end, stamp 0), with
@@ -217,17 +149,22 @@ __device__ __forceinline__ void node_to_window(const uint32_t* buf, uint32_t cap
   q[8 * stride] = t[8 * (size_t)cap];                   // gmin
 }
 
-// The stronger bound of the expansions: the earliest finish EF of every
-// unfinished tool, in index (topological) order -- a running CPU tool its end
-// time, a running GPU tool T + ceil(r / 1024), any other tool the latest of T
-// and its unfinished predecessors' EF, plus its duration in its mode (the
-// least over the modes if open) -- and the makespan is at least the largest
-// EF and the serial-queue sum of lower_bound().  Every start is no earlier
-// than T and than the ends of its predecessors, and no tool runs faster than
-// its isolated duration, so EF never exceeds the true end.  `ef` is a
-// per-thread column of NT words in shared memory (stride `stride`).  Times fit
-// in 32 bits: T plus the durations of a chain of remaining tools stays below
-// the validated makespan bound.
+// Lower bound on the makespan of every mapping that extends a node whose state
+// `s` is at a checkpoint (before the admission at s.T), with the modes of the
+// tools in `known` given by `dg`.  The earliest finish EF of every unfinished
+// tool, in index (topological) order, is
+//   * a running CPU tool's end time (exact);
+//   * T + ceil(r / 1024) of a running GPU tool with r work units left: f[k] >=
+//     f[1] = 1024, and the model rounds GPU progress down and completion times up;
+//   * of any other tool the latest of T and its unfinished predecessors' EF, plus
+//     its duration in its mode (c, g + x or l + g + x; min(c, g + x) if open).
+// No tool starts before T or before its predecessors end, so EF never exceeds
+// the true end, and the makespan is at least the largest EF.  Queued tools run
+// one at a time, so it is also at least T + the sum of the remaining durations of
+// the unfinished tools known to be queued.  `ef` is a per-thread column of NT
+// words in shared memory (stride `stride`).  Times fit in 32 bits: T plus the
+// durations of a chain of remaining tools stays below the validated makespan
+// bound.
 template <int NT, typename TB>
 __device__ __forceinline__ uint32_t forward_bound(const State<NT>& s, const TB& tb, const TreeConsts& tc, Digits dg,
                                                   uint32_t known, uint32_t* ef, uint32_t stride) {

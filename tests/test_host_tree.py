@@ -1,8 +1,9 @@
 """The tree search's node logic, built for the host, against the oracle (no GPU).
 
-tests/host_tree.cpp compiles bf_tree.cuh -- the constants, the sources-first renumbering, node
-expansion and its bound, the leaf re-test, the leaf window and the leaf enumeration with its tie
-rule, the code the tree kernels run -- with g++ and walks the tree depth first.  Its optimum
+tests/host_tree.cpp compiles bf_tree.cuh -- the constants, the sources-first renumbering, the
+start from the first tools' modes, node expansion and its bound, the leaf tools' modes within the
+bound, the leaf window and the leaf runs with their tie rule, the code the tree kernels run --
+with g++ and walks the tree depth first.  Its optimum
 (lowest makespan, ties to the lowest canonical index) must equal the oracle's full enumeration
 in both spaces, pruned from no incumbent and from the optimum's own makespan (the tightest bound
 that keeps the optimum), and unpruned.  The GPU tests check the kernels' level loop on the
@@ -35,17 +36,27 @@ def tree():
                     os.path.join(ROOT, "include"), "-o", out, os.path.join(HERE, "host_tree.cpp")], check=True)
     lib = ctypes.CDLL(out)
     lib.host_tree.argtypes = [ctypes.POINTER(bf.Desc), ctypes.c_uint32, ctypes.c_uint32, ctypes.c_uint32,
-                              ctypes.c_void_p]
+                              ctypes.c_uint32, ctypes.c_void_p]
     lib.host_tree.restype = ctypes.c_int
 
-    def run(scn, space, prune=True, bound=INF):
+    def run(scn, space, prune=True, bound=INF, d0=0):
         res = np.zeros(6, np.uint64)
-        assert lib.host_tree(ctypes.byref(bf.to_desc(scn)), space, int(prune), bound, res.ctypes.data) == 0
+        assert lib.host_tree(ctypes.byref(bf.to_desc(scn)), space, int(prune), bound, d0, res.ctypes.data) == 0
         ms, idx = int(res[0]), int(res[1])
         best = (idx, ms) if ms != 2 ** 64 - 1 else (-1, INF)
         return best, res[2:].tolist()
     lib.host_unpruned_steps.argtypes = [ctypes.POINTER(bf.Desc), ctypes.c_uint32, ctypes.c_int]
     lib.host_unpruned_steps.restype = ctypes.c_uint64
+    lib.host_leaf_modes.argtypes = [ctypes.POINTER(bf.Desc), ctypes.c_uint32, ctypes.c_uint32, ctypes.c_void_p,
+                                    ctypes.c_void_p]
+    lib.host_leaf_modes.restype = ctypes.c_uint64
+
+    def leaf_modes(scn, space, bound):
+        count = np.zeros(2, np.uint64)
+        wrong = lib.host_leaf_modes(ctypes.byref(bf.to_desc(scn)), space, bound, count[:1].ctypes.data,
+                                    count[1:].ctypes.data)
+        return wrong, int(count[0]), int(count[1])
+    run.leaf_modes = leaf_modes
     run.unpruned_steps = lambda scn, space, fresh: lib.host_unpruned_steps(ctypes.byref(bf.to_desc(scn)), space, fresh)
     return run
 
@@ -83,7 +94,7 @@ def test_tree_node_logic_random_dags(tree):
         full = oracle.search(scn, THREADS)
         binary = oracle.search_binary(scn, THREADS)
         for space, want in ((3, full), (2, binary)):
-            got, st = tree(scn, space)
+            got, st = tree(scn, space, d0=t % 4)
             assert got == want, (t, scn, space, got, want, st)
             seen.add(("renumbered", st[2]))
             if want[0] >= 0:
@@ -134,7 +145,7 @@ def test_tree_node_logic_standard_workloads(tree):
         scn = S.config(cfg)
         for space, want in ((3, oracle.search(scn, THREADS)), (2, oracle.search_binary(scn, THREADS))):
             for bound in (INF, want[1]):
-                got, st = tree(scn, space, True, bound)
+                got, st = tree(scn, space, True, bound, d0=8 if space == 3 else 13)  # as the library starts
                 assert got == want, (cfg, space, bound, got, want, st)
             if cfg == 2:
                 assert st[2] == 1
@@ -184,3 +195,25 @@ def test_unpruned_search_simulates_every_mapping_to_its_end(tree, n, joined):
         for space in (3, 2):
             steps = tree.unpruned_steps(scn, space, 1)
             assert tree.unpruned_steps(scn, space, 0) == steps > 0, (t, space)
+
+
+@pytest.mark.parametrize("n", [1, 3, 5, 6, 9])
+@pytest.mark.parametrize("joined", [False, True])
+def test_leaf_modes_keep_every_mapping_within_the_bound(tree, n, joined):
+    """The leaf tools' modes at every leaf node, from bounds at, above and below the optimum and none: each kept
+    combination listed once, and every combination whose makespan is within the bound among them."""
+    rng = np.random.default_rng(50 + n)
+    fewer = 0
+    for t in range(6):
+        scn = S.random_small(rng, n, edge_p=(0.1, 0.4)[t % 2], tight=bool(t % 3), contention=bool(t % 4),
+                             max_time=(5, 60)[t // 3])
+        if joined and n > 1:
+            scn = _with_last_waiting(scn, n)
+        if t % 3 == 2 and n > 3 and not joined:
+            scn = _with_late_sources(rng, scn, n)
+        for space, opt in ((3, oracle.search(scn)[1]), (2, oracle.search_binary(scn)[1])):
+            for bound in (opt, opt + opt // 4, max(opt - 1, 1), INF):
+                wrong, listed, combos = tree.leaf_modes(scn, space, bound)
+                assert wrong == 0, (t, space, bound)
+                fewer += listed < combos
+    assert fewer > 0

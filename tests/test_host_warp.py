@@ -84,8 +84,7 @@ def _layered(n, seed):
     return S.Scenario(n, pred, c, g, x, [S._load_from_vram(v) for v in m], m, 24576, S.slowdown_linear(kmax=n))
 
 
-@pytest.mark.parametrize("n,seed", [(11, 0), (12, 1), (13, 3)])
-@pytest.mark.parametrize("parts", [2, 5, 16])
+@pytest.mark.parametrize("n,seed,parts", [(11, 0, 5), (11, 0, 16), (12, 1, 2), (12, 1, 5), (12, 1, 16), (13, 3, 2)])
 def test_leaf_tasks_while_the_bound_improves(warp, n, seed, parts):
     """The best makespan improves between the tasks of a node group, at every place among them (from 5 % above the
     optimum to the optimum): the optimum is found all the same, and the tasks simulate as many combinations in all as
