@@ -397,3 +397,21 @@ def random_segmented(rng: np.random.Generator, n: int, *, seg_max: int = 6, edge
             m = sum(1 << u for u in range(lo, v) if rng.uniform() < edge_p)
             pred[v] = m or (1 << lo)
     return Scenario(**{**base.to_dict(), "pred_mask": pred})
+
+
+def with_blocked_source(scn: Scenario, *, before_last: bool = False) -> Scenario:
+    """``scn`` with one more tool that waits for nothing, runs 1 us on the CPU and
+    fits no GPU mode.  No barrier cuts the DAG any more, so the tree search runs
+    its tree; yet the tool only ever runs beside the others without touching the
+    GPU, so the optimum is that of ``scn`` with a 0 digit added.  It is numbered
+    last, or ``before_last`` the last tool, which then waits for it too (for
+    scenarios whose last tool waits for every other one)."""
+    n, at = scn.n, scn.n - 1 if before_last else scn.n
+    d = scn.to_dict()
+    for name, v in (("pred_mask", 0), ("cpu_us", 1), ("gpu_us", 1), ("xfer_us", 0), ("load_us", 0),
+                    ("vram_mib", scn.vram_budget_mib + 1)):
+        d[name] = d[name][:at] + [v] + d[name][at:]
+    if before_last:
+        d["pred_mask"][n] |= 1 << at
+    f = scn.slowdown_q10
+    return Scenario(**{**d, "n": n + 1, "slowdown_q10": f + [f[-1]] * max(0, n + 2 - len(f))})

@@ -119,6 +119,37 @@ def test_tree_wide_workloads(name):
             assert res.modes == S.mapping_modes(res.index, scn.n)
 
 
+def _uncut_cases():
+    """(name, scenario without a barrier, optimum of the full space, of the binary one) from the segment rule on the
+    scenario before the added source."""
+    def both(base, before_last):
+        for binary in (False, True):
+            i, ms = segments.search(base, binary=binary, threads=THREADS)
+            yield (i % 3 ** (base.n - 1) + i // 3 ** (base.n - 1) * 3 ** base.n if before_last else i), ms
+    rng = np.random.default_rng(31)
+    for n in (20, 21, 24, 27, 29, 31):
+        base = S.random_segmented(rng, n, seg_max=int(rng.choice([4, 6, 8])), tight=bool(n % 2),
+                                  max_time=int(rng.choice([20, 2000])))
+        yield (f"segmented{n}", S.with_blocked_source(base), *both(base, False))
+    base = S.wide28()
+    assert base.pred_mask[27] and segments.bounds(base)[-1] == (27, 28)  # the last tool waits for every other one
+    yield ("wide28", S.with_blocked_source(base), *both(base, False))
+    yield ("wide28 joined", S.with_blocked_source(base, before_last=True), *both(base, True))
+
+
+def test_tree_wide_without_barriers():
+    """The tree's kernels at 21 to 32 tools: segmented DAGs and the 28-tool workload with a source that no barrier
+    passes (its last tool waiting for every other one, or not), both spaces, from no hint and from the optimum."""
+    for name, scn, *want in _uncut_cases():
+        with bf.create_scenario(scn) as h:
+            for space, w in zip((bf.SPACE_FULL, bf.SPACE_BINARY), want):
+                for hint in (None, w[0]):
+                    res, st = bf.search_tree(h, space, True, hint)
+                    assert _pair(res) == w, (name, space, hint, res, st, w)
+                    assert st["launches"] > 2, (name, space, st)  # cut scenarios take one
+        assert oracle.evaluate(scn, want[0][0]) == want[0][1]
+
+
 def test_tree_full_enumeration_of_32_tool_binary_space():
     """Every binary mapping of the 32-tool workload (2^32, less those under infeasible prefixes)
     simulated: the same optimum as the pruned search."""
