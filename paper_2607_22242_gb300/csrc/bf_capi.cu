@@ -438,12 +438,13 @@ bool segment_tables(const bf_scenario* scn, uint32_t** table) {
 }
 
 // Whether a search of `count` mappings (not the whole space) of a scenario with
-// a lane-tree record runs on it: from an eighth of the space on.  Every root is
-// simulated whatever the range, so smaller ranges are the search kernel's
-// (its time, and the lane tree's, at 1/3, 1/9 and 1/27 of the space: 13-tool
-// sparse DAG 167, 87, 48 and 131, 113, 100 us; 14-tool layered DAG 429, 236, 83
-// and 262, 242, 234 us; 16-tool layered DAG 4.15, 3.21, 0.57 and 1.03, 0.83,
-// 0.69 ms; 18-tool layered DAG 17.5, 14.6, 4.9 and 4.2, 3.3, 3.1 ms).
+// a lane-tree record runs on it: from an eighth of the space on.  A range fixes
+// the modes of the last tools, which lie below the roots, so nearly every root
+// overlaps it and is simulated: smaller ranges are the search kernel's (its time,
+// and the lane tree's, at 1/3, 1/9 and 1/27 of the space: 13-tool sparse DAG 167,
+// 87, 48 and 131, 113, 100 us; 14-tool layered DAG 429, 236, 83 and 262, 242, 234
+// us; 16-tool layered DAG 4.15, 3.21, 0.57 and 1.03, 0.83, 0.69 ms; 18-tool layered
+// DAG 17.5, 14.6, 4.9 and 4.2, 3.3, 3.1 ms).
 bool range_on_lanetree(const bf_scenario* scn, uint64_t count) { return count * 8u >= pow3(scn->desc.n); }
 
 // One launch of the search kernel -- or, for the whole space of a scenario

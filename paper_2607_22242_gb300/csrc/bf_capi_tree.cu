@@ -1,7 +1,7 @@
 // bf_capi_tree.cu -- bf_search_tree (include/bf.h): the host side of the tree
-// search, whose kernels are in bf_tree.cu.  The host keeps the level sizes and
-// decides, step by step, which level to pop next; every step that expands
-// nodes waits (bounded) for the count of their surviving children.
+// search, whose kernels are in bf_tree.cu.  The host decides which level to pop
+// next and launches a chain of expansions down to the leaves; it waits (bounded)
+// once per chain, for how many nodes each level has kept.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -138,14 +138,15 @@ int search_tree_impl(const bf_scenario* scn_const, uint32_t space, uint32_t flag
   //    with every combination of the first d0 tools.  A tree of more
   //    leaf-level nodes than the start makes begins with two dives, chains of
   //    kDives[i] nodes per level, whose leaves set the bound; their other nodes
-  //    are then dropped and the search starts over with that bound.  Over 12 layered and sparse DAGs of 8 to 26 tools, dives of
-  //    {256, 2048} nodes took 0.88 times the 8192 of a single dive on average
-  //    ({256, 8192} 0.91, {1024, 8192} 0.92, {1024} 0.95, {64, 8192} 1.06).
-  //    Dives also pay below kPop leaf-level nodes (14 layered tools 0.62 -> 0.37 ms,
-  //    14 sparse ones 0.48 -> 0.36, the binary space of 24 tools 1.01 -> 0.73).
+  //    are then dropped and the search starts over with that bound.  Over both
+  //    spaces of 12 layered and sparse DAGs of 8 to 26 tools (geometric mean of the
+  //    calls): dives of {256, 2048} nodes 0.29 ms, {256} 0.36, {1024} 0.38, {8192}
+  //    0.45.  Dives also pay below kPop leaf-level nodes (14 layered tools
+  //    0.60 -> 0.28 ms, 14 sparse ones 0.46 -> 0.28, the binary space of 24 tools 2.4
+  //    -> 0.59).
   //    With these chains, the leaf modes (bf_tree.cuh node_leaf_modes) and the
-  //    leaf kernel's tasks full searches went from 2.30 to 0.86 ms (18 layered
-  //    tools), 4.06 to 1.4 (20), 7.4 to 1.7 (24) and 6.4 to 1.6 ms (26).
+  //    leaf kernel's tasks full searches went from 2.30 to 0.59 ms (18 layered
+  //    tools), 4.06 to 0.76 (20), 7.4 to about 1.5 (24) and 6.4 to 1.4 ms (26).
   static constexpr uint32_t kDives[] = {256, 2048};
   constexpr uint32_t kStart = 8192;
   // The whole search, not only each wait, is held to the wait limit.

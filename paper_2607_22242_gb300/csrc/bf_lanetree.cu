@@ -16,7 +16,7 @@ constexpr int kLtThreads = (int)kLtLaunchThreads;
 // compiler picks unbounded, same occupancy: batch call 12.86 -> 12.70 ms,
 // 16-tool full search 1.60 -> 1.58 ms.
 constexpr int kLtBlocksPerSm = 5;
-// The wide one-scenario kernel (17 to 20 tools) holds 11 state words per
+// The wide one-scenario kernel (17 to 20 tools) holds 12 state words per
 // checkpoint and 20 per-tool words per lane: 4 blocks fit an SM.
 constexpr int kLtWideBlocksPerSm = 4;
 

@@ -464,8 +464,8 @@ constexpr uint64_t kLtMaxBlocksPerScenario = 1024;
 // root simulates about R[x] events, a level-1 job R[y] - R[x] and a level-2
 // job n - R[y]; each job also costs about half an event to set up.  4096
 // layered 10-tool DAGs (48 checked by enumeration): 2.9 events per mapping
-// against 2.8 for the best split and 4.1 for the prefix/mid/inner split of
-// the other batch kernel.
+// against 2.8 for the best split and 4.1 for the search kernel's prefix/mid/
+// inner split.
 template <typename TB>
 inline void lanetree_levels(const TB& t, uint64_t min_roots, uint32_t* x_out, uint32_t* y_out) {
   const uint32_t n = t.n;

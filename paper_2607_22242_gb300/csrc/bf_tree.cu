@@ -10,13 +10,13 @@
 //                        survivors are appended to the next level's buffer
 //                        (one atomicAdd per warp on the level's count).
 //   tree_leaf_kernel   : one warp per 32 leaf-level nodes (one per lane) and a
-//                        chunk of the combinations of the last D tools' modes,
+//                        part of the combinations of the last D tools' modes,
 //                        walked over the leaf window (tools from the
 //                        lowest one that can still be running at a leaf
 //                        checkpoint; compiled for 8..32 slots), without those
-//                        in which a leaf tool must end too late; per-block best
-//                        (makespan, index) merged into one 16-byte record by
-//                        compare-and-swap.
+//                        in which a leaf tool must end too late for the bound
+//                        the launch began with; per-block best (makespan, index)
+//                        merged into one 16-byte record by compare-and-swap.
 //
 // Level sizes stay on the device: the launches of a chain of levels are sized
 // for the most nodes a level can hold and read how many there are.
@@ -156,16 +156,17 @@ struct LeafShape {
   static constexpr int min_blocks = NW <= 12 ? 4 : NW <= 16 ? 6 : NW <= 24 ? 5 : 4;
 };
 
-// The tasks of the leaf kernel (leaf_task). About kTreeLeafTasks tasks over
-// all nodes (each prepares its nodes anew; a quarter as many left lanes idle: 24
-// tools 2.6 against 2.1 ms), at least 16 combinations each, taken in turn by the
-// grid's warps.  Few nodes are cut finer, down to 2 combinations a task, for about
-// kTreeLeafFill tasks: one warp for each place on the GPU (20 per SM), which
-// otherwise waits for a chain of 16 simulations on an eighth of them (the first
-// dive of an 18-tool search: 24 groups, 384 tasks, 390 us).  Full / binary space
-// before and after: 8 tools 0.18 -> 0.08 / 0.09 -> 0.08 ms, 16 layered tools 0.78
-// -> 0.63 / 0.38 -> 0.18, 18 tools 1.10 -> 0.86 / 0.43 -> 0.22, 20 tools 1.43 ->
-// 1.09 / 0.41 -> 0.23; 2 combinations for all of kTreeLeafTasks: 20 tools 1.55.
+// The tasks of the leaf kernel (leaf_task).  About kTreeLeafTasks tasks over all
+// nodes (each prepares its nodes anew; a quarter as many take as long, within 4 %
+// over 12 DAGs), at least 16 combinations each, taken in turn by the grid's warps.
+// Few nodes are cut finer, down to 2 combinations a task, for about kTreeLeafFill
+// tasks: one warp for each place on the GPU in the 20- and 24-slot forms (5 blocks
+// of 4 warps on each of 152 SMs; up to 12 slots there are 32 places per SM, at 16
+// slots 24, at 32 slots 16), which otherwise waits for a chain of 16 simulations
+// on an eighth of them.  Full / binary space without and with it: 8 tools 0.18 ->
+// 0.085 / 0.09 -> 0.08 ms, 14 layered tools 0.46 -> 0.28 / 0.27 -> 0.11, 16 tools
+// 0.67 -> 0.51 / 0.33 -> 0.12, 18 tools 0.85 -> 0.59 / 0.35 -> 0.14, 20 tools 0.97
+// -> 0.76 / 0.38 -> 0.18.
 constexpr uint32_t kTreeLeafTasks = 16384;
 constexpr uint32_t kTreeLeafFill = 3072;
 

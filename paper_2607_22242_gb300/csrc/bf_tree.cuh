@@ -441,11 +441,13 @@ __device__ __forceinline__ uint32_t read_bound(const uint32_t* bound) {
 // in some, none in most): while the nodes keep about as many each, every lane
 // walks its own node's; else (fewer than 12 times the fullest node's in all) they
 // are dealt to the lanes one by one over all 32 nodes, a lane resuming the state
-// of whichever node its combination belongs to.  A 24-tool layered DAG had 3.3 of
-// 32 lanes at work with every lane on its own node.  Full searches, own nodes only
-// / dealt only / by this rule: 14 layered tools 0.87 / 0.77 / 0.60 ms, 18 tools
-// 1.28 / 1.36 / 1.05, 26 tools 2.13 / 1.92 / 1.80; binary space of 24 tools 1.20 /
-// 5.5 / 1.00 (dealt lanes leave the common path).
+// of whichever node its combination belongs to (and leaving the others' path).
+// Own nodes only / dealt only / by this rule: full searches of 14 layered tools
+// 0.29 / 0.30 / 0.28 ms, 20 tools 0.73 / 0.81 / 0.76, binary space of 24 tools 0.56
+// / 0.70 / 0.59, geometric mean of 24 searches of 8 to 26 tools 0.29 / 0.37 / 0.29;
+// searches with millions of leaf nodes, which keep the whole grid busy, gain by
+// dealing more often than the rule does: 28 tools in 16 GiB 382 / 175 / 420 ms, 32
+// tools 187 / 131 / 230.
 // Modes, totals and that choice depend on the nodes and on bounds->leaf alone, so
 // that the parts of a group are parts of one list whenever they run; the live
 // bound only gives up single runs.

@@ -225,7 +225,7 @@ def test_lanetree_whole_space_records(host):
 
 def test_lanetree_wide_queue_form(host):
     """The wide form of the one-scenario lane tree (four table chunks, 5-bit queue entries in two words,
-    eleven state words per checkpoint), run at small sizes so that every mapping is checked: random DAGs
+    twelve state words per checkpoint), run at small sizes so that every mapping is checked: random DAGs
     of 8-13 tools with small integer times, and 13 tools without edges whose all-queue mapping holds 13
     waiting tools (the second queue word holds the 13th), each against the oracle."""
     rng = np.random.default_rng(94)
