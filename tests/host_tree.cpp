@@ -74,7 +74,7 @@ struct Search {
     if (tc.prune) {
       const uint32_t combos = leaf_mode_combos(modes, tc);
       for (uint32_t k = 0; k < combos; ++k)
-        leaves += leaf_run<NW>(tw, sdw, rtw.data(), tc, slot.data(), 1u, dg, leaf_mode_digits(modes, tc, k), lb, bound)
+        leaves += leaf_run<NW, true>(tw, sdw, rtw.data(), tc, slot.data(), 1u, dg, leaf_mode_digits(modes, tc, k), lb, bound)
                       ? each : 0u;
     } else {
       leaves += each * leaf_combos<NW>(tw, sdw, rtw.data(), tc, slot.data(), 1u, dg, true, 0u, tc.combos / each, lb);
@@ -262,7 +262,7 @@ struct ModeCheck {
     node_to_window<32>(t.node.data(), 1u, 0u, tc.W0, t.tw.n, t.slot.data(), 1u);
     for (uint32_t c = 0; c < ncomb; ++c) {
       LaneBest lb;
-      leaf_run<32>(t.tw, t.sdw, t.rtw.data(), tc, t.slot.data(), 1u, dg, leaf_digits(c, tc.radix, leaf_tools(tc), 0u), lb,
+      leaf_run<32, false>(t.tw, t.sdw, t.rtw.data(), tc, t.slot.data(), 1u, dg, leaf_digits(c, tc.radix, leaf_tools(tc), 0u), lb,
                    kInfeasible);
       wrong += lb.ms != kInfeasible && lb.ms <= bound && !list[c];
     }
