@@ -213,7 +213,8 @@ BF_API int bf_search_pruned(const bf_scenario* scn, uint64_t hint_index, bf_resu
 typedef struct bf_tree_stats {
   uint64_t nodes;         /* prefix nodes created (tools assigned in the search's order), root included */
   uint64_t leaf_nodes;    /* nodes whose last leaf_depth tools were enumerated */
-  uint64_t leaves;        /* mappings simulated to the end (at most leaf_nodes * modes^leaf_depth) */
+  uint64_t leaves;        /* mappings simulated: to the end, or when pruning until past the best makespan known
+                             (at most leaf_nodes * modes^leaf_depth) */
   uint32_t launches;      /* kernel launches */
   uint32_t leaf_depth;    /* tools enumerated below each leaf node */
   uint32_t incumbent_us;  /* the starting bound (0xFFFFFFFF with BF_TREE_NO_PRUNE) */
@@ -240,18 +241,16 @@ typedef struct bf_tree_stats {
  * device, all-gpu_queue); when the tree is large, two narrow dives to the leaves
  * (256, then 2048 nodes per level) tighten it before the search restarts from the
  * root; at the leaves, modes in which a tool would end too late for the bound are
- * not enumerated;
- * better bounds are found as the search proceeds.  space: BF_SPACE_FULL or
+ * not enumerated; better bounds are found as the search proceeds.  space: BF_SPACE_FULL or
  * BF_SPACE_BINARY.
- * flags: 0 or BF_TREE_NO_PRUNE (every mapping of the space is simulated:
- * full enumeration).  `stats` may be NULL.  Allocates level buffers in the
+ * flags: 0 or BF_TREE_NO_PRUNE (every mapping of the space is simulated to
+ * its end: full enumeration).  `stats` may be NULL.  Allocates level buffers in the
  * handle on first use (about 1.7 GB for 32 tools in the full space).  Blocks
  * until the result is on the host.  A pruned search of a scenario cut by
  * barriers into segments of at most 13 tools (see bf_eval_mappings) enumerates
  * each segment on its own instead, in one launch, and adds their optima up
  * (bf_search_pruned does the same); its stats count the segments as nodes and
- * their mappings as leaves.  The whole search, not only each level
- * step, is held to the wait limit (bf_set_wait_timeout_ms): past it the call
+ * their mappings as leaves.  The whole search, not only each wait, is held to the wait limit (bf_set_wait_timeout_ms): past it the call
  * returns BF_ETIMEOUT (an unpruned full space of 28 or more tools takes
  * hours). */
 BF_API int bf_search_tree(const bf_scenario* scn, uint32_t space, uint32_t flags, uint64_t hint_index,
