@@ -631,7 +631,9 @@ inline void lt_sample_events(const bfk::LaneTreeRecord& r, const uint8_t* mode, 
 // last roots of a search leave lanes idle, the more so the fewer a lane runs.
 // Over all splits of 9 layered and sparse DAGs of 12 to 16 tools, timed one by
 // one, that choice is within 4 % of the fastest split on average (1.24x at
-// worst, a 13-tool DAG; with 0.6 / r 6 %).
+// worst, a 13-tool DAG; with 0.6 / r 6 %); over those of 84 more DAGs of 10 to 15
+// tools within 3 % on average, 1.25x to 1.33x on four layered DAGs of 13 and 14
+// tools where it takes one tool too few into the roots.
 // Against levels from events alone with at least two roots per lane: 17-tool
 // layered DAG 9.1 -> 5.3 ms, 16-tool ones 1.59 -> 1.30 and 1.53 -> 1.53 ms,
 // 12-tool layered ones 112 -> 79 and 101 -> 70 us.
@@ -781,9 +783,10 @@ inline void lanetree_list_record(const bfk::TablesT<32>& t, bfk::LaneTreeRecordT
 // and sparse DAG (ratios 18 to 54) and lost up to 1.9 times on chains, spines
 // and fan-outs (3 to 15), whose narrow windows make the search kernel's events
 // cheap; with 12 to 15 tools it won up to 3.7 times or tied, but for fan-outs
-// of 14 and 15 tools (up to 7 % slower); with 10 and 11 tools, where most lanes
+// of 14 and 15 tools (7 to 26 % slower); with 10 and 11 tools, where most lanes
 // have no root, it won up to 2.2 times on layered and sparse DAGs (1.6 to 3.0
-// and 3.0 to 4.3; two ties) and lost on the others (up to 1.0 and 1.9).  On 59
+// and 3.0 to 4.3; two ties) and lost on the others (up to 1.0 and 1.9), of which
+// 11-tool fan-outs are sent to it all the same (33 -> 46 us).  On 59
 // more DAGs of other seeds the rule's choice took 1.5 % longer than the faster
 // kernel on average.
 inline bool lanetree_preferred(const bfk::Tables& rt, const bfk::Plan& rp, const bfk::Tables& rw, double lt_cost) {
